@@ -361,7 +361,7 @@ bool bones_alloc(emu_handle* h) {
   if (dry || h->nfb > 0)
     ok = ok && h->get(h->frowptr, n + 1) && h->get(h->fcol, fnnz) && h->get(h->fval, fnnz) && h->get(h->fldinv, n) &&
          h->get(h->fin_fixed, n) && h->get(h->zeta, 16 * n) && h->get(h->fdt, 3 * kMaxFreeBones) &&
-         h->get(h->phi_fin, 16 * n) && h->get(h->Einv_fin, 256);
+         h->get(h->phi_fin, 16 * n) && h->get(h->Einv_fin, 256) && h->get(h->phit_fin, 16 * n);
   return ok;
 }
 
@@ -639,6 +639,9 @@ int final_setup_device(emu_handle* h) {
       for (int j = 0; j < 16; ++j) Ei[16 * i + j] += Ev[16 * i + k] * Ev[16 * j + k] / lk;
   }
   BONE_CK(cudaMemcpyAsync(h->Einv_fin, Ei.data(), 256 * 8, cudaMemcpyHostToDevice, h->st));
+  const std::vector<double> T = coarse_root(Eg, Ev);
+  BONE_CK(cudaMemcpyAsync(h->small, T.data(), 256 * 8, cudaMemcpyHostToDevice, h->st));
+  BONE_CK(launch_phit(n, h->phi_fin, h->small, h->phit_fin, h->st));
   BONE_CK(cudaStreamSynchronize(h->st));
   return EMU_OK;
 }
@@ -757,6 +760,7 @@ int bones_final_solve(emu_handle* h) {
     a.dinv = h->fldinv;
     a.phi = h->phi_fin;
     a.Einv = h->Einv_fin;
+    a.phit = h->phit_fin;
     a.max_iter = std::max(20000, 4 * h->prm.pcg_max);
     BONE_CK(cudaMemsetAsync(e64, 0, 24 * n, h->st));
     BONE_CK(launch_pcg<double>(3, a, h->grid_pcg3, h->st));

@@ -157,7 +157,7 @@ extern "C" int emu_fiber_field(int64_t n_verts, const double* rest_pos, int64_t 
   double *d_val = dm.get<double>(nnz), *d_dinv = dm.get<double>(n), *d_b = dm.get<double>(3 * n),
          *d_x = dm.get<double>(3 * n), *d_r = dm.get<double>(3 * n), *d_u = dm.get<double>(3 * n),
          *d_w = dm.get<double>(3 * n), *d_p = dm.get<double>(3 * n), *d_s = dm.get<double>(3 * n),
-         *d_part = dm.get<double>((size_t)grid * (4 * 3 + 3 * kModes)), *d_D = dm.get<double>(9 * m),
+         *d_part = dm.get<double>((size_t)std::max(grid, device_sms()) * 64), *d_D = dm.get<double>(9 * m),
          *d_out = dm.get<double>(3 * m);
   int4* d_tet = dm.get<int4>(m);
   GridBarrier* d_bar = dm.get<GridBarrier>(1);

@@ -20,6 +20,7 @@ namespace emu {
 // A is overwritten (its diagonal holds the eigenvalues), V receives the
 // eigenvectors as columns.
 void host_jacobi_eig(std::vector<double>& A, std::vector<double>& V, int N);
+std::vector<double> coarse_root(const std::vector<double>& E, const std::vector<double>& V);
 
 struct DevBuf {
   void* p;
@@ -79,6 +80,7 @@ struct emu_handle {
   double* phi64 = nullptr;
   float* phi32 = nullptr;
   double* Einv = nullptr;
+  double* phit64 = nullptr;  // 16 x n: Phi T, T T^T = Einv (coarse space of the FP64 CG)
   double* lam_add = nullptr;  // F-form: Phi^T K Phi (48 x 48) and 48 zeros, the capacitance's addend
   bool coarse_ready = false;
   // register-resident FP32 CG: exchange buffer, partial sums, launch shape
@@ -161,7 +163,7 @@ struct emu_handle {
   uint8_t *jfree = nullptr, *jmask = nullptr;
   int32_t *frowptr = nullptr, *fcol = nullptr;
   double *fval = nullptr, *fldinv = nullptr, *zeta = nullptr, *fdt = nullptr;
-  double *phi_fin = nullptr, *Einv_fin = nullptr;  // coarse space of the final solve's CG
+  double *phi_fin = nullptr, *Einv_fin = nullptr, *phit_fin = nullptr;  // coarse space of the final solve's CG
   uint8_t* fin_fixed = nullptr;
   int64_t fnnz = 0;
   BoneArgs bargs() const;
@@ -295,6 +297,8 @@ struct emu_handle {
     a.relres_out = nullptr;
     a.phi = coarse_ready ? phi64 : nullptr;
     a.Einv = coarse_ready ? Einv : nullptr;
+    a.phit = coarse_ready ? phit64 : nullptr;
+    a.bar_clean = true;
     return a;
   }
   PcgArgsT<float> pcg32(const float* rhs, float* x, double tol) {

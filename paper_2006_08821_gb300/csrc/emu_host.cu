@@ -92,6 +92,20 @@ void emu::host_jacobi_eig(std::vector<double>& A, std::vector<double>& V, int N)
 }
 
 
+// T (16 x 16, row-major) with T T^T the pseudo-inverse of a 16 x 16 matrix,
+// from its eigenvalues (diagonal of E) and eigenvectors (columns of V).
+std::vector<double> emu::coarse_root(const std::vector<double>& E, const std::vector<double>& V) {
+  double emax = 0.0;
+  for (int i = 0; i < 16; ++i) emax = std::max(emax, E[17 * i]);
+  std::vector<double> T(256, 0.0);
+  for (int k = 0; k < 16; ++k) {
+    const double lk = E[17 * k];
+    if (!(lk > 1e-12 * emax)) continue;
+    for (int i = 0; i < 16; ++i) T[16 * i + k] = V[16 * i + k] / std::sqrt(lk);
+  }
+  return T;
+}
+
 namespace {
 
 uint64_t splitmix64(uint64_t& x) {
@@ -494,8 +508,9 @@ int autotune(emu_handle* h) {
     }
     set_cg_degree(h, best);
   }
-  // rows per block of the FP64 CG
-  if (cg64(h)) {
+  // rows per block of the FP64 CG's generic kernel (smaller systems run pcg64_kernel, whose shape follows from n)
+  int g64 = 0, rows64 = 0;
+  if (cg64(h) && !pcg64_shape(h->n, h->sms, &g64, &rows64)) {
     int best = -1;
     {
       std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -680,6 +695,9 @@ int build_modes(emu_handle* h) {
       for (int j = 0; j < 16; ++j) Ei[16 * i + j] += Ev[16 * i + k] * Ev[16 * j + k] / lk;
   }
   EMU_CK(cudaMemcpyAsync(h->Einv, Ei.data(), 256 * 8, cudaMemcpyHostToDevice, h->st));
+  const std::vector<double> root = coarse_root(Eg, Ev);
+  EMU_CK(cudaMemcpyAsync(h->small, root.data(), 256 * 8, cudaMemcpyHostToDevice, h->st));
+  EMU_CK(launch_phit(n, h->phi64, h->small, h->phit64, h->st));
   if (h->mixed && h->rpt32 > 0)
     EMU_CK(launch_aphi32(n, h->rowptr, h->col, h->val32, h->phi32, h->aphi32, h->st));
   if (h->cg_part) {  // the coarse rows in the partition order of the pipelined CG
@@ -729,7 +747,7 @@ bool alloc_device(emu_handle* h, int64_t nnz) {
   } else
     ok = ok && h->get(h->gam64, 48 * m) && h->get(h->y64, 9 * m) && h->get(h->d64, 9 * m) && h->get(h->Uw64, 54 * m);
   ok = ok && h->get(h->pr, 16 * n) && h->get(h->pu, 16 * n) && h->get(h->pw, 16 * n) && h->get(h->pp, 16 * n) &&
-       h->get(h->ps, 16 * n) && h->get(h->scratch16, 32 * n) && h->get(h->phi64, 16 * n) && h->get(h->Einv, 256);
+       h->get(h->ps, 16 * n) && h->get(h->scratch16, 32 * n) && h->get(h->phi64, 16 * n) && h->get(h->Einv, 256) && h->get(h->phit64, 16 * n);
   if (h->mixed) {
     ok = ok && h->get(h->phi32, 16 * n) && h->get(h->ug32, 2 * n) && h->get(h->part32, 128 * (int64_t)h->sms) &&
          h->get(h->sync32, 96) && h->get(h->aphi32, 16 * n);
@@ -804,6 +822,7 @@ bool acap_view(const emu_handle* h, AcapView* v) {
   v->ldinv = h->ldinv;
   v->phi = h->coarse_ready ? h->phi64 : nullptr;
   v->Einv = h->coarse_ready ? h->Einv : nullptr;
+  v->phit = h->coarse_ready ? h->phit64 : nullptr;
   v->q0 = h->q0;
   v->grid_pcg = h->grid_pcg3;
   v->pcg_max = h->prm.pcg_max;
@@ -1181,7 +1200,8 @@ int emu_create(const emu_mesh_desc* desc, const emu_params* params, const emu_al
            cudaStreamSynchronize(h->st) == cudaSuccess;
     }
   }
-  if (!ok || cudaMemsetAsync(h->sc, 0, sizeof(DevScalars), h->st) != cudaSuccess) {
+  if (!ok || cudaMemsetAsync(h->sc, 0, sizeof(DevScalars), h->st) != cudaSuccess ||
+      cudaMemsetAsync(h->bar, 0, sizeof(GridBarrier), h->st) != cudaSuccess) {
     h->release();
     delete h;
     return fail(EMU_ERR_CUDA, "upload failed");

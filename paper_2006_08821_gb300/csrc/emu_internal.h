@@ -75,6 +75,7 @@ struct AcapView {
   const double* ldinv;
   const double* phi;     // null when the coarse space is not built
   const double* Einv;
+  const double* phit;
   const double* q0;      // rest-state solution q*(I)
   int grid_pcg;
   int pcg_max;

@@ -187,6 +187,9 @@ extern "C" int emu_acap_solve_noalloc(emu_handle* h, const double* F_device, dou
   a.relres_out = nullptr;
   a.phi = v.phi;
   a.Einv = v.Einv;
+  a.phit = v.phit;
+  int g64 = 0, rows = 0;
+  if (pcg64_shape(v.n, v.sms, &g64, &rows)) a.partials = vw;  // its 64 sums per 32 rows or more fit in w, p, s, which it leaves free
   e = launch_pcg<double>(3, a, grid, st);
   if (e != cudaSuccess) return noalloc_fail(EMU_ERR_CUDA, "launching the CG kernel", e);
   int hc[4] = {0, 0, 0, 0};

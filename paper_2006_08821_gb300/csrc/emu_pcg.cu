@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "emu_internal.h"
 #include "emu_pcg.h"
 
@@ -490,7 +492,19 @@ int pcg_max_grid(int nrhs, int64_t n) {
   return (int)(g < 1 ? 1 : g);
 }
 
+int device_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  return sms;
+}
+
 template <typename T> cudaError_t launch_pcg(int nrhs, const PcgArgsT<T>& args, int grid, cudaStream_t st) {
+  if constexpr (std::is_same_v<T, double>) {
+    int g64 = 0, rows = 0;
+    if (nrhs == 3 && (!args.phi || args.phit) && pcg64_shape(args.n, device_sms(), &g64, &rows))
+      return launch_pcg64(args, g64, rows, st);
+  }
   cudaError_t e = cudaMemsetAsync(args.bar, 0, sizeof(GridBarrier), st);
   if (e != cudaSuccess) return e;
   if (nrhs == 3) {

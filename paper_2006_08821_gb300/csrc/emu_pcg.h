@@ -7,11 +7,20 @@
 
 namespace emu {
 
+// Barrier words in device memory: the generic kernel's (reset by the host
+// before each launch), then those of pcg64_kernel (each on its own line, zero
+// between launches).
 struct GridBarrier {
   unsigned int count;
   unsigned int gen;
   int err;
-  int pad;
+  unsigned int pad0[13];
+  unsigned int v_count;
+  unsigned int pad1[15];
+  unsigned int v_done;
+  unsigned int pad2[15];
+  unsigned int v_err;
+  unsigned int pad3[15];
 };
 
 // Vectors are vertex-major with nrhs values per vertex (x[v * nrhs + j]).
@@ -30,7 +39,7 @@ template <typename T> struct PcgArgsT {
   T* w;
   T* p;
   T* s;
-  double* partials;  // grid * 4 * nrhs
+  double* partials;  // grid * (4 nrhs + 16 nrhs); pcg64_kernel: 64 per block of its own grid
   GridBarrier* bar;
   double tol;        // stop when ||r_j|| <= tol ||b_j|| for every column j
   int max_iter;
@@ -41,10 +50,21 @@ template <typename T> struct PcgArgsT {
   double* relres_out;  // final ||r_j|| / ||b_j|| per column (may be null)
   const T* phi;        // n x 16 coarse basis (null: Jacobi only; 3 columns only)
   const double* Einv;  // 16 x 16 (pseudo-)inverse of Phi^T L Phi
+  const T* phit = nullptr;  // 16 x n: Phi T with T T^T = Einv, mode-major (FP64; null where phi is)
+  bool bar_clean = false;   // bar's v_ words are zero: no memset before a launch of pcg64_kernel
   unsigned long long wait_ns = kWaitLimitNs;  // limit of each grid-barrier wait
 };
 
 int pcg_max_grid(int nrhs, int64_t n);
+// The FP64 CG with its rows on chip (emu_pcg64.cu), which launch_pcg<double>
+// takes for three columns when the shape exists (n <= 320 rows per SM) and
+// the coarse space, if any, comes with phit. args.u holds the exchanged
+// vector (3 n); r, w, p and s are unused.
+bool pcg64_shape(int64_t n, int sms, int* grid, int* rows);
+cudaError_t launch_pcg64(const PcgArgsT<double>& args, int grid, int rows, cudaStream_t st);
+int device_sms();  // multiprocessors of the current device
+// phit of a coarse basis phi (n x 16) and T (16 x 16, row-major, device)
+cudaError_t launch_phit(int64_t n, const double* phi, const double* T, double* out, cudaStream_t st);
 template <typename T> cudaError_t launch_pcg(int nrhs, const PcgArgsT<T>& args, int grid, cudaStream_t st);
 
 constexpr int kPcg32Threads = 256;  // threads per block of the FP32 CG kernels

@@ -1,0 +1,467 @@
+// FP64 conjugate gradient of the coupling solve (Eq. 4, three right-hand
+// sides) with every row's state on chip: the FP64 path's dq solves and exact
+// re-solves, the mixed path's solves with bones, the allocation-free solve
+// and the fiber field.
+//
+// The iteration is the generic kernel's (pcg_kernel in emu_pcg.cu:
+// Chronopoulos-Gear CG, Jacobi plus the additive coarse space). What bounds it
+// on these systems (400 to 50,000 rows) is latency: two grid barriers, one L2
+// gather and one sum over the blocks per iteration, and the FP64 pipe, which
+// issues two FMAs per cycle and SM. So:
+//   * a warp owns one column of 32 rows (three warps per 32 rows), so a row's
+//     chains are 16 products long, a warp's reduction carries 19 values
+//     instead of 57, and no lane idles;
+//   * x, r, p, s, u, w stay in registers; the matrix (16 entries per row) and
+//     the coarse rows stay in shared memory, one copy for the three columns;
+//     only u goes through L2;
+//   * the coarse basis comes as Phi' = Phi T with T T^T = E^-1, so
+//     M = D^-1 + Phi' Phi'^T needs no 16 x 16 product between the reduction
+//     and the next u;
+//   * as few as 32 rows per block while a block per SM suffices: the FP64 work
+//     of a row (about 165 FMAs per iteration) is what more SMs share, and the
+//     barrier costs little more with 152 blocks than with 5. Rows per block
+//     grow in steps of 32 once n exceeds 32 per SM (up to 320);
+//   * the barrier is a release-add and an acquire poll on one counter that
+//     the last block to leave zeroes, so no memset precedes a launch;
+//   * one division on the path from the sums to alpha: with den the last
+//     denominator, beta g / alpha = beta^2 den.
+// Measured on one GB300 against the generic kernel (whole calls): coupling
+// solve of 19,833 rows 4.87 -> 2.08 ms; two-bone arm of 692 rows (45 CG
+// iterations per Newton iteration) 434 -> 226 ms a solve; box beam of 425 rows
+// in FP64 94 -> 72 ms; 6,080-tet unit in FP64 82 -> 67 ms.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <mutex>
+
+#include "emu_internal.h"
+#include "emu_pcg.h"
+
+namespace emu {
+
+namespace {
+
+constexpr int NR = 3;
+constexpr int kEll = 16;        // entries of a matrix row held in shared memory
+constexpr int kRed = 20;        // values a warp reduces: gamma, delta, rr, bb, 16 modes
+constexpr int kPart = 64;       // doubles per block in the partial sums
+constexpr int kMaxRows = 320;   // rows per block at most (960 threads)
+constexpr int kNV = 12 + NR * kModes;  // gamma, delta, rr, bb (3 columns each), Phi'^T w
+
+__device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Grid barrier on bar->v_count (arrivals of the launch so far). Bounded: a
+// wait that runs out raises v_err, every other waiter sees it and leaves.
+__device__ __forceinline__ bool vbar(GridBarrier* bar, unsigned& epoch, int* s_flag, unsigned long long wait_ns) {
+  __syncthreads();
+  epoch += 1u;
+  if (threadIdx.x == 0) {
+    red_release_add(&bar->v_count, 1u);
+    const unsigned target = gridDim.x * epoch;
+    int bad = 0;
+    unsigned long long spins = 0, t0 = 0;
+    while (ld_acquire(&bar->v_count) < target) {
+      ++spins;
+      if ((spins & 63u) == 0u) {
+        if (*((volatile unsigned*)&bar->v_err)) {
+          bad = 1;
+          break;
+        }
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > wait_ns || spins > kWaitSpinCap) {
+          bad = 1;
+          atomicExch(&bar->v_err, 1u);
+          break;
+        }
+      }
+    }
+    *s_flag = bad;
+  }
+  __syncthreads();
+  return *s_flag == 0;
+}
+
+// The last block to leave zeroes the words for the next launch.
+__device__ __forceinline__ void vbar_exit(GridBarrier* bar) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&bar->v_done, 1u) + 1u == gridDim.x) {
+      atomicExch(&bar->v_count, 0u);
+      atomicExch(&bar->v_err, 0u);
+      atomicExch(&bar->v_done, 0u);
+    }
+  }
+}
+
+// Halving butterfly of C values (a power of two) over one warp in a fixed
+// order: lane l ends with the sum of value (l * C / 32) in v[0].
+template <int C, int O>
+__device__ __forceinline__ void warp_halve(double* v, int lane) {
+  if constexpr (C >= 2) {
+    constexpr int H = C / 2;
+    const bool hi = (lane & O) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double send = hi ? v[i] : v[H + i];
+      const double keep = hi ? v[H + i] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    if constexpr (O > 1) warp_halve<H, O / 2>(v, lane);
+  } else {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+    if constexpr (O > 1) warp_halve<1, O / 2>(v, lane);
+  }
+}
+
+}  // namespace
+
+// blockDim.x = max(256, 3 rows); warp w < 3 rows / 32 owns column w % 3 of
+// the rows 32 (w / 3) .. + 31 of the block; further warps help with the sums.
+template <int MAXT, bool COARSE>
+__global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int rows) {
+  constexpr int NC = COARSE ? kModes : 0;
+  __shared__ double s_red[(kMaxRows / 32) * NR * kRed];
+  __shared__ double s_grp[16 * kPart];
+  __shared__ double s_rho[NR * kModes], s_sig[NR * kModes];
+  __shared__ double s_al[NR], s_be[NR];
+  __shared__ int s_act[NR], s_zero[NR];
+  __shared__ int s_flag;
+  extern __shared__ double dyn[];
+  double* sVal = dyn;                        // [kEll][rows]
+  double* sPhi = sVal + kEll * rows;         // [16][rows] when COARSE
+  int32_t* sCol = reinterpret_cast<int32_t*>(sPhi + NC * rows);  // [kEll][rows]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = gridDim.x;
+  const int64_t n = a.n;
+  const int64_t r0 = (int64_t)blockIdx.x * rows;
+  const int nrow = (int)(n - r0 < rows ? n - r0 : rows);
+  const int grp = warp / NR, j = warp % NR;  // row group and column of this warp
+  const int lr = grp * 32 + lane;            // row of this thread in the block
+  const bool data = grp * 32 < rows;         // a warp with rows
+  const bool own = data && lr < nrow;
+  const int64_t v = r0 + (own ? lr : 0);
+  unsigned epoch = 0;
+  double* __restrict__ ug = a.u;  // [3][n]
+  double* __restrict__ part = a.partials;
+
+  int cnt = 0;
+  int32_t e0 = 0, e1 = 0;
+  if (own) {
+    e0 = __ldg(a.rowptr + v);
+    e1 = __ldg(a.rowptr + v + 1);
+    cnt = e1 - e0;
+  }
+  // the three warps of a row group fill its matrix entries and coarse rows
+  if (data) {
+    for (int t = j; t < kEll; t += NR) {
+      sVal[t * rows + lr] = own && t < cnt ? __ldg(a.val + e0 + t) : 0.0;
+      sCol[t * rows + lr] = own && t < cnt ? __ldg(a.col + e0 + t) : (int32_t)v;
+    }
+    if constexpr (COARSE)
+      for (int m = j; m < kModes; m += NR) sPhi[m * rows + lr] = own ? __ldg(a.phit + (size_t)m * n + v) : 0.0;
+  }
+  const double di = own ? __ldg(a.dinv + v) : 0.0;
+  const double bv = own ? a.b[v * NR + j] : 0.0;
+  double x = own ? a.x[v * NR + j] : 0.0;
+  __syncthreads();
+
+  // one entry of A z, z element c at z[c * stride + j * plane]
+  auto spmv = [&](const double* z, int64_t stride, int64_t plane) -> double {
+    if (!own) return 0.0;
+    const double* zj = z + j * plane;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    constexpr int GW = MAXT > 512 ? 8 : 16;  // gathers in flight
+#pragma unroll
+    for (int t0 = 0; t0 < kEll; t0 += GW) {
+      double zz[GW];
+#pragma unroll
+      for (int t = 0; t < GW; ++t) zz[t] = t0 + t < cnt ? __ldcg(zj + sCol[(t0 + t) * rows + lr] * stride) : 0.0;
+#pragma unroll
+      for (int t = 0; t < GW; ++t) acc[t & 3] = fma(sVal[(t0 + t) * rows + lr], zz[t], acc[t & 3]);
+    }
+    for (int32_t e = e0 + kEll; e < e1; e += 4) {  // long rows
+      double av[4], zz[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const bool on = e + t < e1;
+        av[t] = on ? __ldg(a.val + e + t) : 0.0;
+        zz[t] = on ? __ldcg(zj + __ldg(a.col + e + t) * stride) : 0.0;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) acc[t] = fma(av[t], zz[t], acc[t]);
+    }
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  };
+  // u = D^-1 r + Phi' rho
+  auto precond = [&](double r) -> double {
+    double acc[4] = {di * r, 0.0, 0.0, 0.0};
+    if constexpr (COARSE) {
+      if (data) {
+#pragma unroll
+        for (int m = 0; m < kModes; ++m) acc[m & 3] = fma(sPhi[m * rows + lr], s_rho[j * kModes + m], acc[m & 3]);
+      }
+    }
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  };
+  // block sums of d4 (gamma, delta, rr, bb of this thread) and Phi'^T y, written as this block's partials
+  auto reduce = [&](const double (&d4)[4], double y) {
+    if (data) {
+      double t4[4] = {d4[0], d4[1], d4[2], d4[3]};
+      warp_halve<4, 16>(t4, lane);
+      if ((lane & 7) == 0) s_red[warp * kRed + (lane >> 3)] = t4[0];
+      if constexpr (COARSE) {
+        double t[kModes];
+#pragma unroll
+        for (int m = 0; m < kModes; ++m) t[m] = sPhi[m * rows + lr] * y;
+        warp_halve<kModes, 16>(t, lane);
+        if ((lane & 1) == 0) s_red[warp * kRed + 4 + (lane >> 1)] = t[0];
+      }
+    }
+    __syncthreads();
+    if (tid < 12 + NR * NC) {
+      // value q < 12: item q / 3 of column q % 3; then mode (q - 12) % 16 of column (q - 12) / 16
+      const int jj = tid < 12 ? tid % NR : (tid - 12) / kModes;
+      const int item = tid < 12 ? tid / NR : 4 + (tid - 12) % kModes;
+      double t = 0.0;
+      for (int g = 0; g * 32 < rows; ++g) t += s_red[(g * NR + jj) * kRed + item];
+      __stcg(part + (size_t)blockIdx.x * kPart + tid, t);
+    }
+  };
+  // sum over the blocks in a fixed order: groups of 64 threads take every
+  // NG-th block, eight loads in flight; thread k < kNV returns value k
+  auto gather_sums = [&]() -> double {
+    const int k = tid & (kPart - 1), g = tid / kPart, NG = (int)blockDim.x / kPart;
+    if (k < 12 + NR * NC && g < NG) {
+      double t = 0.0;
+      int b = g;
+      for (; b + 7 * NG < G; b += 8 * NG) {
+        double l[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) l[q] = __ldcg(part + (size_t)(b + q * NG) * kPart + k);
+        t += ((l[0] + l[1]) + (l[2] + l[3])) + ((l[4] + l[5]) + (l[6] + l[7]));
+      }
+      if (b < G) {  // the rest, loads in flight too
+        double l[7];
+#pragma unroll
+        for (int q = 0; q < 7; ++q) l[q] = b + q * NG < G ? __ldcg(part + (size_t)(b + q * NG) * kPart + k) : 0.0;
+        t += ((l[0] + l[1]) + (l[2] + l[3])) + ((l[4] + l[5]) + l[6]);
+      }
+      s_grp[g * kPart + k] = t;
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (tid < kPart)
+      for (int gg = 0; gg < NG; ++gg) t += s_grp[gg * kPart + tid];
+    return t;
+  };
+
+  // ---- r = b - A x (x in place: it is written back only after two barriers)
+  double r = bv - spmv(a.x, NR, 1);
+  if (!own) r = 0.0;
+  if constexpr (COARSE) {  // rho = Phi'^T r
+    const double z4[4] = {0.0, 0.0, 0.0, 0.0};
+    reduce(z4, r);
+    if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+    const double t = gather_sums();
+    if (tid >= 12 && tid < kNV) s_rho[tid - 12] = t;
+    __syncthreads();
+  }
+  {
+    double u = precond(r);
+    if (own) __stcg(ug + j * n + v, u);
+    if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+    double w = spmv(ug, 1, n);
+    {
+      const double d4[4] = {r * u, w * u, r * r, bv * bv};
+      reduce(d4, w);
+    }
+    if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+    // scalars of column l in lane l of warp 0
+    double sg = 0.0, sden = 0.0, sig_ = 0.0, sthr = 0.0, sbb = 0.0, srr = 0.0, sal = 0.0;
+    int sact = 0;
+    double t = gather_sums();
+    if (warp == 0) {
+      const double g = t, dl = __shfl_sync(0xffffffffu, t, (lane + 3) & 31), rr = __shfl_sync(0xffffffffu, t, (lane + 6) & 31),
+                   bb = __shfl_sync(0xffffffffu, t, (lane + 9) & 31);
+      if (lane < NR) {
+        sbb = bb;
+        srr = rr;
+        sthr = a.tol * a.tol * bb;
+        sg = g;
+        sden = dl;
+        sig_ = 1.0 / g;
+        sact = (rr <= sthr || !(dl > 0.0)) ? 0 : 1;
+        sal = sact ? g / dl : 0.0;
+        s_al[lane] = sal;
+        s_be[lane] = 0.0;
+        s_act[lane] = sact;
+        s_zero[lane] = bb == 0.0;
+      }
+    }
+    __syncthreads();
+    if (COARSE && tid >= 12 && tid < kNV) {
+      const int q = tid - 12;
+      s_sig[q] = t;
+      if (s_act[q / kModes]) s_rho[q] -= s_al[q / kModes] * t;
+    }
+    __syncthreads();
+    double p = u, s = w;
+    if (s_zero[j]) x = 0.0;  // zero right-hand side: x = 0 exactly
+    int it = 0;
+    bool all_done = !(s_act[0] || s_act[1] || s_act[2]);
+    while (!all_done && it < a.max_iter) {
+      ++it;
+      if (s_act[j]) {
+        const double al = s_al[j];
+        x = fma(al, p, x);
+        r = fma(-al, s, r);
+      }
+      u = precond(r);
+      if (own) __stcg(ug + j * n + v, u);
+      if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+      w = spmv(ug, 1, n);
+      {
+        const double d4[4] = {r * u, w * u, r * r, 0.0};
+        reduce(d4, w);
+      }
+      if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+      t = gather_sums();
+      if (warp == 0) {
+        const double g = t, dl = __shfl_sync(0xffffffffu, t, (lane + 3) & 31),
+                     rr = __shfl_sync(0xffffffffu, t, (lane + 6) & 31);
+        if (lane < NR && sact) {
+          srr = rr;
+          const double be = g * sig_;
+          const double den = dl - be * be * sden;
+          if (rr <= sthr || !(den > 0.0)) {  // converged, or breakdown: stop this column
+            sact = 0;
+            s_act[lane] = 0;
+          } else {
+            s_be[lane] = be;
+            s_al[lane] = g / den;
+            sig_ = 1.0 / g;
+            sden = den;
+          }
+        }
+      }
+      __syncthreads();
+      if (COARSE && tid >= 12 && tid < kNV) {  // sigma = Phi'^T w + beta sigma, rho -= alpha sigma
+        const int q = tid - 12, c = q / kModes;
+        if (s_act[c]) {
+          const double sg2 = fma(s_be[c], s_sig[q], t);
+          s_sig[q] = sg2;
+          s_rho[q] -= s_al[c] * sg2;
+        }
+      }
+      if (s_act[j]) {
+        const double be = s_be[j];
+        p = fma(be, p, u);
+        s = fma(be, s, w);
+      }
+      all_done = !(s_act[0] || s_act[1] || s_act[2]);
+      __syncthreads();
+    }
+    if (own) a.x[v * NR + j] = x;
+    if (blockIdx.x == 0 && warp == 0) {
+      if (lane == 0) {
+        if (a.iters_out) atomicAdd(a.iters_out, it);
+        if (a.fail_out && !all_done) atomicExch(a.fail_out, 1);
+        if (a.last_iters) *a.last_iters = it;
+      }
+      if (lane < NR && a.relres_out) a.relres_out[lane] = sbb > 0.0 ? sqrt(srr / sbb) : 0.0;
+    }
+  }
+  vbar_exit(a.bar);
+  return;
+timeout:
+  if (tid == 0 && a.timeout_out) atomicExch(a.timeout_out, 1);
+  vbar_exit(a.bar);
+}
+
+namespace {
+size_t pcg64_smem(int rows, bool coarse) {
+  return (size_t)rows * (8 * kEll + 4 * kEll + (coarse ? 8 * kModes : 0));
+}
+
+template <int MAXT, bool C>
+cudaError_t launch64(const PcgArgsT<double>& args, int rows, int grid, int threads, cudaStream_t st) {
+  const size_t smem = pcg64_smem(rows, C);
+  if (smem > 40 * 1024) {  // with the static arrays above the default 48 KB: opt in once per device
+    static bool set[64] = {false};
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!set[dev]) {
+      e = cudaFuncSetAttribute(pcg64_kernel<MAXT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)pcg64_smem(MAXT / NR, C));
+      if (e != cudaSuccess) return e;
+      set[dev] = true;
+    }
+  }
+  PcgArgsT<double> a = args;
+  int r = rows;
+  void* params[] = {(void*)&a, (void*)&r};
+  return cudaLaunchCooperativeKernel((const void*)pcg64_kernel<MAXT, C>, dim3(grid), dim3(threads), params, smem, st);
+}
+
+template <bool C> cudaError_t pick64(const PcgArgsT<double>& a, int rows, int grid, cudaStream_t st) {
+  const int threads = std::max(256, NR * rows);
+  if (threads <= 288) return launch64<288, C>(a, rows, grid, threads, st);
+  if (threads <= 480) return launch64<480, C>(a, rows, grid, threads, st);
+  return launch64<960, C>(a, rows, grid, threads, st);
+}
+}  // namespace
+
+// Rows per block: the smallest multiple of 32 that needs at most one block
+// per SM; false above 320 (n > 320 per SM: the generic kernel).
+bool pcg64_shape(int64_t n, int sms, int* grid, int* rows) {
+  if (sms < 1 || n < 1) return false;
+  const int64_t r = std::max<int64_t>(1, (n + 32 * (int64_t)sms - 1) / (32 * (int64_t)sms)) * 32;
+  if (r > kMaxRows) return false;
+  *rows = (int)r;
+  *grid = (int)((n + r - 1) / r);
+  return true;
+}
+
+cudaError_t launch_pcg64(const PcgArgsT<double>& args, int grid, int rows, cudaStream_t st) {
+  if (!args.bar_clean) {
+    const cudaError_t e = cudaMemsetAsync(args.bar, 0, sizeof(GridBarrier), st);
+    if (e != cudaSuccess) return e;
+  }
+  return args.phit ? pick64<true>(args, rows, grid, st) : pick64<false>(args, rows, grid, st);
+}
+
+// out[k n + v] = sum_l phi[v][l] T[l][k]: the coarse basis with T T^T = E^-1, mode-major
+__global__ void __launch_bounds__(256) k_phit(int64_t n, const double* __restrict__ phi, const double* __restrict__ T,
+                                              double* __restrict__ out) {
+  __shared__ double sT[kModes * kModes];
+  for (int e = threadIdx.x; e < kModes * kModes; e += blockDim.x) sT[e] = T[e];
+  __syncthreads();
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * kModes; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = i / n, v = i % n;
+    double acc = 0.0;
+    for (int l = 0; l < kModes; ++l) acc = fma(phi[v * kModes + l], sT[l * kModes + k], acc);
+    out[i] = acc;
+  }
+}
+
+cudaError_t launch_phit(int64_t n, const double* phi, const double* T, double* out, cudaStream_t st) {
+  const int grid = (int)std::min<int64_t>(std::max<int64_t>(1, (n * kModes + 255) / 256), 4096);
+  k_phit<<<grid, 256, 0, st>>>(n, phi, T, out);
+  return cudaGetLastError();
+}
+
+}  // namespace emu
