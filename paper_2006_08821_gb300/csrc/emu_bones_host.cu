@@ -667,13 +667,16 @@ const double* bones_cap_addend(const emu_handle* h) {
   return h->nfb > 0 ? h->cadd : h->cconst;
 }
 
+// blocks of the direction kernel in use
+static int dir_grid(const emu_handle* h) { return h->mixed ? h->grid_tet : h->grid_t64; }
+
 void bones_before_dir(emu_handle* h) {
   if (h->nfb == 0) return;
-  launch_bone_dir(h->bargs(), h->z, h->part_dir + h->grid_tet, h->st);
+  launch_bone_dir(h->bargs(), h->z, h->part_dir + dir_grid(h), h->st);
   h->launches += 1;
 }
 
-int dir_partial_count(const emu_handle* h) { return h->grid_tet + (h->nfb > 0 ? 1 : 0); }
+int dir_partial_count(const emu_handle* h) { return dir_grid(h) + (h->nfb > 0 ? 1 : 0); }
 
 void joints_project(emu_handle* h, double* x64, float* x32) {
   if (h->npts == 0) return;

@@ -288,6 +288,7 @@ __global__ void __launch_bounds__(128) k_grad_fform(TetArgs<double> a) {
   }
   block_reduce_write<1>(acc, a.partials + blockIdx.x);
   if (bad) atomicExch(&a.sc->nonfinite, 1);
+  grad_finish(a.sc, a.partials);
 }
 
 // ------------------------------------------------------------ capacitance --
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(128) k_grad_fform(TetArgs<double> a) {
 // 3r .. 3r+2. The block sums -Yh^T Yh (the Woodbury term of Eq. 12) and
 // B y = sum_i w_i (G_i Phi)^T y_i: By[16r+j] = sum_i w_i sum_b y[r][b] gam_j[b].
 __global__ void __launch_bounds__(256) k_syrk_fform(TetArgs<double> a, double* __restrict__ cpart) {
-  constexpr int CH = 8;  // tets per chunk
+  constexpr int CH = kSyrk64Chunk;  // tets per chunk
   constexpr int KR = CH * 9;
   __shared__ double sY[KR][kK + 1];
   __shared__ double sL[CH][kFformL];
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(256) k_syrk_fform(TetArgs<double> a, double* _
 // d = -(y + alpha w H^-1 v), v = (G_i Phi) z; g . d; corners of w G^T d.
 __global__ void __launch_bounds__(128) k_dir_fform(TetArgs<double> a) {
   __shared__ double sz[kK];
-  if (threadIdx.x < kK) sz[threadIdx.x] = a.z[threadIdx.x];
+  for (int k = threadIdx.x; k < kK; k += blockDim.x) sz[k] = a.z[k];
   __syncthreads();
   const int64_t m = a.m;
   double acc[1] = {0.0};
@@ -435,7 +436,8 @@ __global__ void __launch_bounds__(128) k_dir_fform(TetArgs<double> a) {
 // (ln det(I + sigma M), M = F^-1 d, through log1p of its polynomial), and
 // the ACAP part's two coefficients alpha w <D, dD>, alpha w |dD|^2 with
 // D = G q - F, dD = G dq - d.
-__global__ void __launch_bounds__(128) k_ls_fform(TetArgs<double> a, double rho) {
+__global__ void __launch_bounds__(128) k_ls_fform(TetArgs<double> a, LsSelect sel) {
+  const double rho = sel.rho;
   const int64_t m = a.m;
   const double s0 = a.sc->sigma_start;
   double acc[kLsNV];
@@ -507,13 +509,16 @@ __global__ void __launch_bounds__(128) k_ls_fform(TetArgs<double> a, double rho)
     }
   }
   block_reduce_write<kLsNV>(acc, a.partials + (size_t)blockIdx.x * kLsNV);
+  ls_finish(a.sc, a.partials, sel);
 }
 
 // ------------------------------------------------------------ update ------
-__global__ void __launch_bounds__(256) k_update_fform(TetArgs<double> a) {
+__global__ void __launch_bounds__(256) k_update_fform(TetArgs<double> a, double* __restrict__ q) {
   const double sig = a.sc->sigma;
   if (sig == 0.0) return;
   const int64_t m = a.m;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < 3 * a.n; k += (int64_t)gridDim.x * blockDim.x)
+    q[k] += sig * a.dq[k];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
 #pragma unroll
     for (int k = 0; k < 9; ++k) a.R[k * m + i] += sig * a.d[k * m + i];
@@ -577,16 +582,20 @@ __global__ void __launch_bounds__(128) k_eval_fform(const double* F, const doubl
 static int fform_grid(int64_t m, int threads) { return (int)(m > 0 ? (m + threads - 1) / threads : 1); }
 
 void launch_rhs_fform(const TetArgs<double>& a, int grid, cudaStream_t st) { k_rhs_fform<<<grid, 256, 0, st>>>(a); }
-void launch_grad_fform(const TetArgs<double>& a, int grid, cudaStream_t st) { k_grad_fform<<<grid, 128, 0, st>>>(a); }
+void launch_grad_fform(const TetArgs<double>& a, int grid, int threads, cudaStream_t st) {
+  k_grad_fform<<<grid, threads, 0, st>>>(a);
+}
 void launch_syrk_fform(const TetArgs<double>& a, int grid, double* cpart, cudaStream_t st) {
   k_syrk_fform<<<grid, 256, 0, st>>>(a, cpart);
 }
-void launch_dir_fform(const TetArgs<double>& a, int grid, cudaStream_t st) { k_dir_fform<<<grid, 128, 0, st>>>(a); }
-void launch_ls_fform(const TetArgs<double>& a, int grid, double rho, cudaStream_t st) {
-  k_ls_fform<<<grid, 128, 0, st>>>(a, rho);
+void launch_dir_fform(const TetArgs<double>& a, int grid, int threads, cudaStream_t st) {
+  k_dir_fform<<<grid, threads, 0, st>>>(a);
 }
-void launch_update_fform(const TetArgs<double>& a, int grid, cudaStream_t st) {
-  k_update_fform<<<grid, 256, 0, st>>>(a);
+void launch_ls_fform(const TetArgs<double>& a, int grid, int threads, const LsSelect& sel, cudaStream_t st) {
+  k_ls_fform<<<grid, threads, 0, st>>>(a, sel);
+}
+void launch_update_fform(const TetArgs<double>& a, int grid, double* q, cudaStream_t st) {
+  k_update_fform<<<grid, 256, 0, st>>>(a, q);
 }
 void launch_fform_to_Rs(int64_t m, const double* F, double* R, double* s, cudaStream_t st) {
   k_fform_to_Rs<<<fform_grid(m, 128), 128, 0, st>>>(m, F, R, s);

@@ -20,14 +20,14 @@ constexpr int kFformL = 45;
 // holding F (9m, component-major k * m + i), a.Uw the factors (45m), and
 // a.g, a.y, a.d, a.gam, a.contrib, a.z, a.partials as there. No bones.
 void launch_rhs_fform(const TetArgs<double>& a, int grid, cudaStream_t st);
-void launch_grad_fform(const TetArgs<double>& a, int grid, cudaStream_t st);
+void launch_grad_fform(const TetArgs<double>& a, int grid, int threads, cudaStream_t st);
 // cpart as for launch_syrk, holding the partials of -alpha sum w^2
 // (G Phi)^T H^-1 (G Phi): C = Lambda + that sum takes Lambda = Phi^T K Phi
 // as the addend of launch_cap_solve.
 void launch_syrk_fform(const TetArgs<double>& a, int grid, double* cpart, cudaStream_t st);
-void launch_dir_fform(const TetArgs<double>& a, int grid, cudaStream_t st);
-void launch_ls_fform(const TetArgs<double>& a, int grid, double rho, cudaStream_t st);
-void launch_update_fform(const TetArgs<double>& a, int grid, cudaStream_t st);
+void launch_dir_fform(const TetArgs<double>& a, int grid, int threads, cudaStream_t st);
+void launch_ls_fform(const TetArgs<double>& a, int grid, int threads, const LsSelect& sel, cudaStream_t st);
+void launch_update_fform(const TetArgs<double>& a, int grid, double* q, cudaStream_t st);
 // R and s (component-major, like the rotation/stretch state) of the polar
 // decomposition F = R S of each tet's F.
 void launch_fform_to_Rs(int64_t m, const double* F, double* R, double* s, cudaStream_t st);

@@ -172,6 +172,7 @@ struct emu_handle {
 
   // launch shapes
   int grid_tet = 1, grid_syrk = 1, grid_pcg3 = 1, grid_pcg16 = 1;
+  int grid_t64 = 1, threads_t64 = 128;  // FP64 per-tet kernels (tet64_shape)
   int grid_tet4 = 1;  // one wave of the 4-blocks-per-SM mixed gradient and line-search kernels
 
   // profiling: event pairs per phase, resolved at the next host sync

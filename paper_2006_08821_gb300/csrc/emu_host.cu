@@ -762,7 +762,8 @@ bool alloc_device(emu_handle* h, int64_t nnz) {
     }
   }
   h->grid_tet = (int)std::min<int64_t>(std::max<int64_t>(1, (m + 127) / 128), 8 * (int64_t)h->sms);
-  h->grid_syrk = (int)std::min<int64_t>(std::max<int64_t>(1, (m + 23) / 24), 2 * (int64_t)h->sms);
+  h->grid_syrk = (int)std::min<int64_t>(std::max<int64_t>(1, (m + kSyrk64Chunk - 1) / kSyrk64Chunk), 2 * (int64_t)h->sms);
+  tet64_shape(m, h->sms, &h->grid_t64, &h->threads_t64);
   h->grid_tet4 = (int)std::min<int64_t>(std::max<int64_t>(1, (m + 127) / 128), 4 * (int64_t)h->sms);
   h->grid_pcg3 = pcg_max_grid(3, n);
   h->grid_pcg16 = pcg_max_grid(16, n);
@@ -770,8 +771,9 @@ bool alloc_device(emu_handle* h, int64_t nnz) {
   const int g3max = h->prm.autotune ? std::max<int>(h->grid_pcg3, (int)std::min<int64_t>((n + 63) / 64, h->sms))
                                     : h->grid_pcg3;
   const int pcg_part = std::max(g3max * (4 * 3 + 3 * kModes), h->grid_pcg16 * 64);  // per-block partials
-  const int64_t gpart = std::max<int64_t>(h->grid_tet * (int64_t)kLsNV, 256 * (int64_t)(2 * h->sms + 1));
-  ok = ok && h->get(h->part_grad, gpart) && h->get(h->part_dir, h->grid_tet + 1) && h->get(h->part_ls, (h->grid_tet + kBoneLsBlocks) * kLsNV) &&
+  const int64_t gpart = std::max<int64_t>(std::max(h->grid_tet, h->grid_t64) * (int64_t)kLsNV, 256 * (int64_t)(2 * h->sms + 1));
+  ok = ok && h->get(h->part_grad, gpart) && h->get(h->part_dir, std::max(h->grid_tet, h->grid_t64) + 1) &&
+       h->get(h->part_ls, (std::max(h->grid_tet, h->grid_t64) + kBoneLsBlocks) * kLsNV) &&
        h->get(h->part_pcg, std::max<int64_t>(pcg_part, 256 * (int64_t)(2 * h->sms + 1))) &&
        h->get(h->cpart, std::max<int64_t>(h->grid_syrk, std::max(kTcBlocksPerSM, kSyrk05BlocksPerSM) * (int64_t)h->sms) *
                             (kCapEntries + kK)) && h->get(h->z, kK) && h->get(h->cfull, kCapEntries + kK) && h->get(h->small, 256) &&
@@ -1367,16 +1369,11 @@ int enqueue_grad(emu_handle* h) {
     launch_split_disp(h->n, h->q, h->Qrest, h->uh32, h->ul32, h->st);
     launch_grad_mixed(h->margs(), h->grid_tet4, h->st);
   } else if (h->fform) {
-    launch_grad_fform(h->args<double>(), h->grid_tet, h->st);
+    launch_grad_fform(h->args<double>(), h->grid_t64, h->threads_t64, h->st);
   } else {
-    launch_grad<double>(h->args<double>(), h->grid_tet, h->st);
+    launch_grad<double>(h->args<double>(), h->grid_t64, h->threads_t64, h->st);
   }
   h->ph_end(EMU_PHASE_GRAD, h->mixed ? 2 : 1);
-  if (!h->mixed) {  // the mixed gradient kernel reduces ||g||^2 in its last block
-    h->ph_begin();
-    launch_reduce_grad(h->part_grad, h->grid_tet, h->sc, nullptr, nullptr, h->st);
-    h->ph_end(EMU_PHASE_SMALL, 1);
-  }
   if (h->nfb > 0) {  // the free bones' virtual elements (Sec. 3.3)
     h->ph_begin();
     bones_after_grad(h);
@@ -1411,7 +1408,7 @@ int enqueue_direction(emu_handle* h) {
   launch_cap_solve(h->cpart, syrk_blocks, h->cfull, h->z, h->sc, h->mixed && !h->has_bones, h->st,
                    h->fform ? h->lam_add : bones_cap_addend(h));
   bones_before_dir(h);
-  h->ph_end(EMU_PHASE_SMALL, 2);
+  h->ph_end(EMU_PHASE_SMALL, 1);
   h->ph_begin();
   if (h->mixed) {
     MixArgs ad = am;
@@ -1421,9 +1418,9 @@ int enqueue_direction(emu_handle* h) {
     TetArgs<double> ad = a64;
     ad.partials = h->part_dir;
     if (h->fform)
-      launch_dir_fform(ad, h->grid_tet, h->st);
+      launch_dir_fform(ad, h->grid_t64, h->threads_t64, h->st);
     else
-      launch_dir<double>(ad, h->grid_tet, h->st);
+      launch_dir<double>(ad, h->grid_t64, h->threads_t64, h->st);
   }
   h->ph_end(EMU_PHASE_DIR, 1);
   EMU_CK(cudaGetLastError());
@@ -1440,39 +1437,34 @@ int enqueue_step(emu_handle* h) {
   if (rc) return rc;
   // Armijo line search (Algorithm 1)
   h->ph_begin();
+  LsSelect sel;  // the line-search kernel's last block selects the step
+  sel.dir_partials = h->part_dir;
+  sel.nblk_dir = dir_partial_count(h);
+  sel.sigma0 = h->sigma0_now;
+  sel.rho = h->prm.ls_rho;
+  sel.c_armijo = h->prm.ls_c;
+  const int ls_grid = h->mixed ? h->grid_tet4 : h->grid_t64;
+  if (h->nfb > 0) {  // the free bones' terms in FP64, after the kernel's own partials
+    double* bone_part = h->part_ls + (size_t)ls_grid * kLsNV;
+    if (h->mixed)
+      launch_bone_ls(h->bargs(), h->dq32, h->prm.ls_rho, bone_part, h->st);
+    else
+      launch_bone_ls(h->bargs(), h->dq, h->prm.ls_rho, bone_part, h->st);
+    sel.nblk_extra = kBoneLsBlocks;
+  }
   if (h->mixed) {
     MixArgs al = am;
     al.partials = h->part_ls;
-    LsSelect sel;  // the line-search kernel's last block selects the step
-    sel.dir_partials = h->part_dir;
-    sel.nblk_dir = dir_partial_count(h);
-    sel.sigma0 = h->sigma0_now;
-    sel.rho = h->prm.ls_rho;
-    sel.c_armijo = h->prm.ls_c;
-    if (h->nfb > 0) {  // the free bones' terms in FP64, after the kernel's own partials
-      launch_bone_ls(h->bargs(), h->dq32, h->prm.ls_rho, h->part_ls + (size_t)h->grid_tet4 * kLsNV, h->st);
-      sel.nblk_extra = kBoneLsBlocks;
-    }
-    launch_ls_mixed(al, h->grid_tet4, sel, h->st);
-    h->ph_end(EMU_PHASE_LS, 1);
+    launch_ls_mixed(al, ls_grid, sel, h->st);
   } else {
     TetArgs<double> al = a64;
     al.partials = h->part_ls;
-    int nls = h->grid_tet;
-    if (h->nfb > 0) {  // the free bones' terms, after the per-tet partials
-      launch_bone_ls(h->bargs(), h->dq, h->prm.ls_rho, h->part_ls + (size_t)h->grid_tet * kLsNV, h->st);
-      nls += kBoneLsBlocks;
-    }
     if (h->fform)
-      launch_ls_fform(al, h->grid_tet, h->prm.ls_rho, h->st);
+      launch_ls_fform(al, ls_grid, h->threads_t64, sel, h->st);
     else
-      launch_ls<double>(al, h->grid_tet, h->prm.ls_rho, h->st);
-    h->ph_end(EMU_PHASE_LS, 1);
-    h->ph_begin();
-    launch_ls_select(h->part_dir, dir_partial_count(h), h->part_ls, nls, h->sc, h->sigma0_now, h->prm.ls_rho,
-                     h->prm.ls_c, h->st);
-    h->ph_end(EMU_PHASE_SMALL, 1);
+      launch_ls<double>(al, ls_grid, h->threads_t64, sel, h->st);
   }
+  h->ph_end(EMU_PHASE_LS, 1);
   h->ph_begin();
   if (h->mixed) {
     launch_update_mixed(am, h->grid_tet, h->st);
@@ -1483,12 +1475,11 @@ int enqueue_step(emu_handle* h) {
       launch_update_verts_f(h->n, h->sc, h->dq32, h->q, h->st);
   } else {
     if (h->fform)
-      launch_update_fform(a64, h->grid_tet, h->st);
+      launch_update_fform(a64, h->grid_tet, h->q, h->st);
     else
-      launch_update_tets<double>(a64, h->grid_tet, h->st);
-    launch_update_verts(h->n, h->sc, h->dq, h->q, h->st);
+      launch_update_tets<double>(a64, h->grid_t64, h->threads_t64, h->q, h->st);
   }
-  h->ph_end(EMU_PHASE_UPDATE, 2);
+  h->ph_end(EMU_PHASE_UPDATE, h->mixed ? 2 : 1);
   EMU_CK(cudaGetLastError());
   return EMU_OK;
 }

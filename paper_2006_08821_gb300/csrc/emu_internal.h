@@ -26,9 +26,9 @@ struct DevScalars {
   int32_t pcg_fail;     // a CG solve hit pcg_max
   int32_t barrier_timeout;
   int32_t nonfinite;    // a non-finite value was produced
-  uint32_t ticket[2];   // blocks done in the current gradient / line-search launch
+  uint32_t ticket[3];   // blocks done in the current gradient / line-search / capacitance launch
 };
-constexpr int kTicketGrad = 0, kTicketLs = 1;
+constexpr int kTicketGrad = 0, kTicketLs = 1, kTicketCap = 2;
 
 // Mesh constants on the device (structure of arrays, index i = tet).
 template <typename T> struct MeshArrays {

@@ -147,20 +147,11 @@ __global__ void __launch_bounds__(128) k_grad(TetArgs<TW> a) {
   }
   block_reduce_write<1>(acc, a.partials + blockIdx.x);
   if (bad) atomicExch(&a.sc->nonfinite, 1);
+  grad_finish(a.sc, a.partials);
 }
 
-template <typename TW> void launch_grad(const TetArgs<TW>& a, int grid, cudaStream_t st) {
-  k_grad<TW><<<grid, 128, 0, st>>>(a);
-}
-
-__global__ void __launch_bounds__(256) k_reduce_grad(const double* partials, int nblk, DevScalars* sc) {
-  __shared__ double tot[1];
-  block_sum_partials<1>(partials, nblk, tot);
-  if (threadIdx.x == 0) sc->gnorm2 = tot[0];
-}
-
-void launch_reduce_grad(const double* partials, int nblk, DevScalars* sc, double*, double*, cudaStream_t st) {
-  k_reduce_grad<<<1, 256, 0, st>>>(partials, nblk, sc);
+template <typename TW> void launch_grad(const TetArgs<TW>& a, int grid, int threads, cudaStream_t st) {
+  k_grad<TW><<<grid, threads, 0, st>>>(a);
 }
 
 // ------------------------------------------------------------ capacitance --
@@ -170,13 +161,17 @@ void launch_reduce_grad(const double* partials, int nblk, DevScalars* sc, double
 // Also B y = sum_i w_i (G_i Phi^T)^T y_i: By[16r+j] = sum_i w_i sum_b y[r][b] gam_j[b].
 template <typename TW>
 __global__ void __launch_bounds__(256) k_syrk(TetArgs<TW> a, double* __restrict__ cpart) {
-  constexpr int CH = sizeof(TW) == 8 ? 8 : 16;  // tets per chunk
+  // tets per chunk: few in FP64, whose pipe takes 10 us per 8 tets, so that
+  // the chunks of a small mesh spread evenly over the SMs (6,080 tets at two
+  // blocks per SM: 10 chunks of 4 on every SM, before 48 or 24 tets)
+  constexpr int CH = sizeof(TW) == 8 ? kSyrk64Chunk : 16;
   constexpr int KR = CH * 6;
   __shared__ TW sY[KR][kK + 1];
   __shared__ TW sU[CH][54];
   __shared__ TW sg[CH][48];
   __shared__ TW sy[CH][9];
   __shared__ double sw[CH];
+  __shared__ TW ssw[CH];  // sqrt(w), once per tet
   const int tid = threadIdx.x;
   int tr = 0, tc = 0;
   const bool tile = lower_tile(tid, tr, tc);  // 5 of the 8 warps issue the product
@@ -205,7 +200,10 @@ __global__ void __launch_bounds__(256) k_syrk(TetArgs<TW> a, double* __restrict_
       const int64_t i = base + tt;
       sy[tt][k] = i < m ? a.y[k * m + i] : TW(0);
     }
-    if (tid < CH) sw[tid] = (base + tid) < m ? a.w[base + tid] : 0.0;
+    if (tid < CH) {
+      sw[tid] = (base + tid) < m ? a.w[base + tid] : 0.0;
+      ssw[tid] = (TW)sqrt(sw[tid]);
+    }
     __syncthreads();
     for (int e = tid; e < CH * 6 * kK; e += 256) {
       const int tt = e / (6 * kK), rem = e % (6 * kK);
@@ -213,7 +211,7 @@ __global__ void __launch_bounds__(256) k_syrk(TetArgs<TW> a, double* __restrict_
       const int r = col >> 4, j = col & 15;
       TW v = sU[tt][9 * k + 3 * r] * sg[tt][3 * j] + sU[tt][9 * k + 3 * r + 1] * sg[tt][3 * j + 1] +
              sU[tt][9 * k + 3 * r + 2] * sg[tt][3 * j + 2];
-      sY[tt * 6 + k][col] = v * (TW)sqrt(sw[tt]);
+      sY[tt * 6 + k][col] = v * ssw[tt];
     }
     __syncthreads();
 #pragma unroll 4
@@ -257,102 +255,155 @@ template <typename TW> void launch_syrk(const TetArgs<TW>& a, int grid, double* 
   k_syrk<TW><<<grid, 256, 0, st>>>(a, cpart);
 }
 
-// One warp per entry of C and B y sums that entry's per-block partials
-// (entry-major, coalesced) with a fixed shuffle tree.
-__global__ void __launch_bounds__(256) k_reduce_cpart(const double* __restrict__ cpart, int nblk, double* __restrict__ cfull,
-                                                      const double* __restrict__ cadd) {
-  const int e = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (e >= kCapEntries + kK) return;
-  double x = 0.0;
-  for (int b = lane; b < nblk; b += 32) x += cpart[(size_t)e * nblk + b];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  if (lane == 0) cfull[e] = cadd ? x + cadd[e] : x;
+// ------------------------------------------- capacitance sum and solve ----
+// 1 / d by Newton's iteration from a hardware estimate (its error is at most
+// an ulp; one step leaves rounding), without a division's range handling.
+__device__ __forceinline__ float pivot_inverse(float d) {
+  if (!(d > 1e-30f && d < 1e30f)) return 1.f / d;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return fmaf(r, fmaf(-d, r, 1.f), r);
+}
+// Newton's iteration for 1 / d from an FP32 start (relative error 1e-7, 1e-14,
+// then rounding): six dependent operations instead of a division's sequence.
+__device__ __forceinline__ double pivot_inverse(double d) {
+  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
+  double r = (double)(1.f / (float)d);
+  r = fma(r, fma(-d, r, 1.0), r);
+  return fma(r, fma(-d, r, 1.0), r);
 }
 
-// Factor C = L L^T (C symmetrised) and solve z = C^-1 (B y), in T arithmetic
+constexpr int kCapLow = kK * (kK + 1) / 2;        // entries of the lower triangle
+constexpr int kCapSums = kCapLow + kK;            // and of B y
+constexpr int kCapNB = 4;                         // columns of a panel
+constexpr int kCapOwn = (kCapSums + 255) / 256;   // entries a thread of the solving block owns
+
+// Sums the per-block partials of C (lower triangle) and B y, one warp per
+// entry (entry-major, coalesced, a fixed shuffle tree), and in the last block
+// to finish factors C = L D L^T and solves z = C^-1 (B y) in T arithmetic
 // (FP64; FP32 for the mixed path, whose C comes from TF32 products).
-// Right-looking Cholesky with all 256 threads and one barrier per column:
-// the column below the diagonal is left unscaled (L_ij = C_ij / sqrt(d_j),
-// d_j the pivot), so each column is a single rank-1 update of the trailing
-// lower triangle, C_ik -= C_ij C_kj / d_j, on a fixed 16 x 16 thread grid.
-// The two triangular solves run in one warp with the right-hand side in
-// registers. In FP64 the pivots' reciprocals and square roots on GB300's
-// narrow FP64 path set its latency.
+//
+// Latency decides here: one block, 48 dependent pivots. Each of the 256
+// threads owns up to five entries of the lower triangle in registers, with
+// B y as row 48, so the forward substitution is part of the factorisation.
+// Per panel of four columns the owners hand the panel to one warp, which
+// factors it with its rows in registers (shuffles instead of barriers), and
+// every thread then applies the four rank-1 updates to its entries: two block
+// barriers per four columns, and the work of the trailing triangle only. The
+// entries are numbered from the last column backwards, so the trailing
+// entries are a prefix and whole warps drop out as it shrinks. In FP64 a warp
+// instruction holds GB300's FP64 pipe for 16 cycles: 9.2e3 cycles for the
+// updates, and the pivots' reciprocals are Newton steps in one warp.
+// Measured per launch pair before (reduction, then a 256-thread factorisation
+// with a barrier and a division per column): FP32 27 us, FP64 95 us a Newton
+// iteration; the fused kernel's figures stand in the kernel table.
 template <typename T>
-__global__ void __launch_bounds__(256) k_cap_solve(const double* __restrict__ cfull, double* z, DevScalars* sc) {
-  __shared__ T C[kK][kK + 1];
-  __shared__ T rinv[kK];  // 1 / sqrt(d_j)
-  __shared__ int s_ok;
-  const int tid = threadIdx.x;
-  const int ti = tid >> 4, tk = tid & 15;
-  for (int e = tid; e < kCapEntries; e += blockDim.x) C[e / kK][e % kK] = (T)cfull[e];
-  if (tid == 0) s_ok = 1;
-  __syncthreads();
-  // unused modes (k_modes < 48) have zero rows: make them identity rows
-  if (tid < kK && cfull[tid * kK + tid] == 0.0) C[tid][tid] = T(1);
-  // symmetrise into the lower triangle
-  for (int e = tid; e < kCapEntries; e += blockDim.x) {
-    const int i = e / kK, j = e % kK;
-    if (j < i) C[i][j] = T(0.5) * (C[i][j] + C[j][i]);
+__global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, int nblk, double* __restrict__ cfull,
+                                             const double* __restrict__ cadd, double* z, DevScalars* sc) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  {
+    const int e = blockIdx.x * 8 + (tid >> 5);
+    if (e < kCapSums) {
+      int src = kCapEntries + (e - kCapLow);  // of cpart: row-major 48 x 48, then B y
+      if (e < kCapLow) {
+        int i = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        while (i * (i + 1) / 2 > e) --i;
+        src = i * kK + (e - i * (i + 1) / 2);
+      }
+      double x = 0.0;
+      for (int b = lane; b < nblk; b += 32) x += cpart[(size_t)src * nblk + b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if (lane == 0) __stcg(cfull + src, cadd ? x + cadd[src] : x);
+    }
   }
-  __syncthreads();
-  for (int j = 0; j < kK; ++j) {
-    T d = C[j][j];
-    if (!(d > T(0))) d = T(1);  // failure is recorded below
-    const T rho = T(1) / d;
+  if (!last_block(&sc->ticket[kTicketCap])) return;
+  __shared__ T sL[kK + 1][kK + 1];      // finished columns of L; row 48: D^-1 L^-1 (B y)
+  __shared__ T sP[kCapNB][kK + 1];      // the panel's columns
+  __shared__ T sW[kCapNB][kK + 1];      // L D of the panel
+  __shared__ int s_ok;
+  // entry t: column 48 - a and row 48 - b with 0 <= b <= a, t = a (a + 1) / 2 + b (a = 0 is unused)
+  int row[kCapOwn], col[kCapOwn];
+  T val[kCapOwn];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int i = j + 1 + ti + 16 * a;
-      if (i >= kK) break;
-      const T cij = C[i][j] * rho;
+  for (int s = 0; s < kCapOwn; ++s) {
+    const int t = 1 + tid + 256 * s;
+    int a = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+    while ((a + 1) * (a + 2) / 2 <= t) ++a;
+    while (a * (a + 1) / 2 > t) --a;
+    col[s] = kK - a;
+    row[s] = kK - (t - a * (a + 1) / 2);
+    val[s] = T(0);
+    if (t <= kCapSums) {
+      const double diag = __ldcg(cfull + col[s] * kK + col[s]);
+      const double v = row[s] < kK ? __ldcg(cfull + row[s] * kK + col[s]) : __ldcg(cfull + kCapEntries + col[s]);
+      val[s] = (T)v;
+      // unused modes (k_modes < 48) have zero rows: identity rows with a zero right-hand side
+      if (diag == 0.0) val[s] = row[s] == col[s] ? T(1) : row[s] == kK ? T(0) : val[s];
+    } else {
+      col[s] = -1;
+    }
+  }
+  if (tid == 0) s_ok = 1;
+  for (int p0 = 0; p0 < kK; p0 += kCapNB) {
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const int k = j + 1 + tk + 16 * b;
-        if (k <= i) C[i][k] -= cij * C[k][j];
+    for (int s = 0; s < kCapOwn; ++s)
+      if (col[s] >= p0 && col[s] < p0 + kCapNB) sP[col[s] - p0][row[s]] = val[s];
+    __syncthreads();
+    if (tid < 32) {
+      // rows p0 + lane and p0 + 32 + lane of the panel
+      const int ra = p0 + lane, rb = ra + 32;
+      T va[kCapNB], vb[kCapNB];
+#pragma unroll
+      for (int q = 0; q < kCapNB; ++q) {
+        va[q] = (ra <= kK && ra >= p0 + q) ? sP[q][ra] : T(0);
+        vb[q] = rb <= kK ? sP[q][rb] : T(0);
+      }
+#pragma unroll
+      for (int p = 0; p < kCapNB; ++p) {
+        T d = __shfl_sync(0xffffffffu, va[p], p);
+        if (!(d > T(0))) {  // not positive definite: recorded, z = 0 below
+          d = T(1);
+          s_ok = 0;
+        }
+        const T ri = pivot_inverse(d);
+        if (ra <= kK) sW[p][ra] = va[p];
+        if (rb <= kK) sW[p][rb] = vb[p];
+#pragma unroll
+        for (int q = p + 1; q < kCapNB; ++q) {
+          const T l = __shfl_sync(0xffffffffu, va[p], q) * ri;
+          va[q] -= va[p] * l;
+          vb[q] -= vb[p] * l;
+        }
+        if (ra <= kK) sL[ra][p0 + p] = va[p] * ri;
+        if (rb <= kK) sL[rb][p0 + p] = vb[p] * ri;
       }
     }
     __syncthreads();
+#pragma unroll
+    for (int s = 0; s < kCapOwn; ++s)
+      if (col[s] >= p0 + kCapNB) {
+#pragma unroll
+        for (int q = 0; q < kCapNB; ++q) val[s] -= sW[q][row[s]] * sL[col[s]][p0 + q];
+      }
   }
-  if (tid < kK) {
-    const T d = C[tid][tid];
-    if (!(d > T(0))) atomicExch(&s_ok, 0);
-    rinv[tid] = d > T(0) ? T(1) / sqrt(d) : T(1);
-  }
-  __syncthreads();
-  if (tid < 32) {
-    const int lane = tid;
+  if (tid < 32) {  // L^T z = y
     const bool has1 = lane + 32 < kK;
-    T x0 = (T)cfull[kCapEntries + lane];
-    T x1 = has1 ? (T)cfull[kCapEntries + lane + 32] : T(0);
-    if (cfull[lane * kK + lane] == 0.0) x0 = T(0);  // unused mode: identity row, zero right-hand side
-    if (has1 && cfull[(lane + 32) * kK + lane + 32] == 0.0) x1 = T(0);
-    // L y = b: y_j = x_j / L_jj, then x_i -= L_ij y_j for i > j
-    for (int j = 0; j < kK; ++j) {
-      const T xj = __shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31);
-      const T yj = xj * rinv[j];
-      const T f = rinv[j] * yj;  // L_ij y_j = C_ij f
-      if (lane == (j & 31)) {
-        if (j < 32) x0 = yj; else x1 = yj;
-      }
-      if (lane > j) x0 -= C[lane][j] * f;
-      if (has1 && lane + 32 > j) x1 -= C[lane + 32][j] * f;
-    }
-    // L^T z = y: z_j = x_j / L_jj, then x_i -= L_ji z_j for i < j
-    for (int j = kK - 1; j >= 0; --j) {
-      const T xj = __shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31);
-      const T zj = xj * rinv[j];
-      if (lane == (j & 31)) {
-        if (j < 32) x0 = zj; else x1 = zj;
-      }
-      if (lane < j) x0 -= C[j][lane] * rinv[lane] * zj;
-      if (has1 && lane + 32 < j) x1 -= C[j][lane + 32] * rinv[lane + 32] * zj;
+    T x0 = sL[kK][lane], x1 = has1 ? sL[kK][lane + 32] : T(0);
+#pragma unroll 4
+    for (int j = kK - 1; j > 0; --j) {
+      const T zj = __shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31);
+      if (lane < j) x0 -= sL[j][lane] * zj;
+      if (has1 && lane + 32 < j) x1 -= sL[j][lane + 32] * zj;
     }
     const int ok = s_ok;
     z[lane] = ok ? (double)x0 : 0.0;
     if (has1) z[lane + 32] = ok ? (double)x1 : 0.0;
-    if (lane == 0) sc->cap_ok = ok ? 1.0 : 0.0;
+    if (lane == 0) {
+      sc->cap_ok = ok ? 1.0 : 0.0;
+      sc->ticket[kTicketCap] = 0u;
+    }
   }
 }
 
@@ -366,11 +417,11 @@ void launch_ls_reset(DevScalars* sc, double sigma0, cudaStream_t st) { k_ls_rese
 void launch_cap_solve(const double* cpart, int nblk, const double* cfull_scratch, double* z, DevScalars* sc,
                       bool fp32_factor, cudaStream_t st, const double* cadd) {
   double* cfull = const_cast<double*>(cfull_scratch);
-  k_reduce_cpart<<<(kCapEntries + kK + 7) / 8, 256, 0, st>>>(cpart, nblk, cfull, cadd);
+  const int grid = (kCapSums + 7) / 8;
   if (fp32_factor)
-    k_cap_solve<float><<<1, 256, 0, st>>>(cfull, z, sc);
+    k_cap<float><<<grid, 256, 0, st>>>(cpart, nblk, cfull, cadd, z, sc);
   else
-    k_cap_solve<double><<<1, 256, 0, st>>>(cfull, z, sc);
+    k_cap<double><<<grid, 256, 0, st>>>(cpart, nblk, cfull, cadd, z, sc);
 }
 
 // ------------------------------------------------------------ direction ---
@@ -378,7 +429,7 @@ void launch_cap_solve(const double* cpart, int nblk, const double* cfull_scratch
 template <typename TW>
 __global__ void __launch_bounds__(128) k_dir(TetArgs<TW> a) {
   __shared__ double sz[kK];
-  if (threadIdx.x < kK) sz[threadIdx.x] = a.z[threadIdx.x];
+  for (int k = threadIdx.x; k < kK; k += blockDim.x) sz[k] = a.z[k];
   __syncthreads();
   const int64_t m = a.m;
   double acc[1] = {0.0};
@@ -432,8 +483,8 @@ __global__ void __launch_bounds__(128) k_dir(TetArgs<TW> a) {
   block_reduce_write<1>(acc, a.partials + blockIdx.x);
 }
 
-template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, cudaStream_t st) {
-  k_dir<TW><<<grid, 128, 0, st>>>(a);
+template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, int threads, cudaStream_t st) {
+  k_dir<TW><<<grid, threads, 0, st>>>(a);
 }
 
 // ------------------------------------------------------------ line search --
@@ -443,7 +494,8 @@ template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, cudaStrea
 // + sigma^2 e2(M) + sigma^3 det M). The ACAP part is the exact quadratic
 // alpha/2 sum w |D + sigma dD|^2 - |D|^2, D = G q - F, dD = G dq - d.
 template <typename TW>
-__global__ void __launch_bounds__(128) k_ls(TetArgs<TW> a, double rho) {
+__global__ void __launch_bounds__(128) k_ls(TetArgs<TW> a, LsSelect sel) {
+  const double rho = sel.rho;
   const int64_t m = a.m;
   const double s0 = a.sc->sigma_start;
   double acc[kLsNV];
@@ -525,30 +577,23 @@ __global__ void __launch_bounds__(128) k_ls(TetArgs<TW> a, double rho) {
     }
   }
   block_reduce_write<kLsNV>(acc, a.partials + (size_t)blockIdx.x * kLsNV);
+  ls_finish(a.sc, a.partials, sel);
 }
 
-template <typename TW> void launch_ls(const TetArgs<TW>& a, int grid, double rho, cudaStream_t st) {
-  k_ls<TW><<<grid, 128, 0, st>>>(a, rho);
-}
-
-__global__ void __launch_bounds__(256) k_ls_select(const double* dir_partials, int nblk_dir, const double* ls_partials,
-                                                    int nblk_ls, DevScalars* sc, double sigma0, double rho, double c_armijo) {
-  ls_select_block(dir_partials, nblk_dir, ls_partials, nblk_ls, sc, sigma0, rho, c_armijo);
-}
-
-void launch_ls_select(const double* dir_partials, int nblk_dir, const double* ls_partials, int nblk_ls,
-                      DevScalars* sc, double sigma0, double rho, double c_armijo, cudaStream_t st) {
-  k_ls_select<<<1, 256, 0, st>>>(dir_partials, nblk_dir, ls_partials, nblk_ls, sc, sigma0, rho, c_armijo);
+template <typename TW> void launch_ls(const TetArgs<TW>& a, int grid, int threads, const LsSelect& sel, cudaStream_t st) {
+  k_ls<TW><<<grid, threads, 0, st>>>(a, sel);
 }
 
 // ------------------------------------------------------------ update ------
 // F' = R S + sigma d; X = R^T F' = S + sigma R^T d is nearly symmetric, so its
 // polar factor Rx is close to I; R' = R Rx, S' = sym(Rx^T X).
 template <typename TW>
-__global__ void __launch_bounds__(128) k_update_tets(TetArgs<TW> a) {
+__global__ void __launch_bounds__(128) k_update_tets(TetArgs<TW> a, double* __restrict__ q) {
   const double sig = a.sc->sigma;
   if (sig == 0.0) return;
   const int64_t m = a.m;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < 3 * a.n; k += (int64_t)gridDim.x * blockDim.x)
+    q[k] += sig * a.dq[k];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     double R[9], sv[6], S[9], d[9], Rtd[9], X[9], Rx[9], Rn[9], Sn[9], sn[6];
 #pragma unroll
@@ -572,8 +617,8 @@ __global__ void __launch_bounds__(128) k_update_tets(TetArgs<TW> a) {
   }
 }
 
-template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, cudaStream_t st) {
-  k_update_tets<TW><<<grid, 128, 0, st>>>(a);
+template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, int threads, double* q, cudaStream_t st) {
+  k_update_tets<TW><<<grid, threads, 0, st>>>(a, q);
 }
 
 __global__ void __launch_bounds__(256) k_update_verts(int64_t n3, const DevScalars* sc, const double* dq, double* q) {
@@ -870,16 +915,16 @@ void launch_compose_F(int64_t m, const double* R, const double* s, double* F, cu
 }
 
 // explicit instantiations
-template void launch_grad<double>(const TetArgs<double>&, int, cudaStream_t);
-template void launch_grad<float>(const TetArgs<float>&, int, cudaStream_t);
+template void launch_grad<double>(const TetArgs<double>&, int, int, cudaStream_t);
+template void launch_grad<float>(const TetArgs<float>&, int, int, cudaStream_t);
 template void launch_syrk<double>(const TetArgs<double>&, int, double*, cudaStream_t);
 template void launch_syrk<float>(const TetArgs<float>&, int, double*, cudaStream_t);
-template void launch_dir<double>(const TetArgs<double>&, int, cudaStream_t);
-template void launch_dir<float>(const TetArgs<float>&, int, cudaStream_t);
-template void launch_ls<double>(const TetArgs<double>&, int, double, cudaStream_t);
-template void launch_ls<float>(const TetArgs<float>&, int, double, cudaStream_t);
-template void launch_update_tets<double>(const TetArgs<double>&, int, cudaStream_t);
-template void launch_update_tets<float>(const TetArgs<float>&, int, cudaStream_t);
+template void launch_dir<double>(const TetArgs<double>&, int, int, cudaStream_t);
+template void launch_dir<float>(const TetArgs<float>&, int, int, cudaStream_t);
+template void launch_ls<double>(const TetArgs<double>&, int, int, const LsSelect&, cudaStream_t);
+template void launch_ls<float>(const TetArgs<float>&, int, int, const LsSelect&, cudaStream_t);
+template void launch_update_tets<double>(const TetArgs<double>&, int, int, double*, cudaStream_t);
+template void launch_update_tets<float>(const TetArgs<float>&, int, int, double*, cudaStream_t);
 template void launch_gamma<double>(int64_t, const int4*, const double*, const double*, double*, cudaStream_t);
 template void launch_gamma<float>(int64_t, const int4*, const double*, const double*, float*, cudaStream_t);
 

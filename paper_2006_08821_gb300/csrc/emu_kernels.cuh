@@ -9,6 +9,28 @@
 
 namespace emu {
 
+// Armijo selection the last block of a line-search kernel performs.
+struct LsSelect {
+  const double* dir_partials;
+  int nblk_dir;
+  double sigma0, rho, c_armijo;
+  // blocks of line-search partials written after the kernel's own (the free
+  // bones' FP64 terms, Sec. 3.3), summed by the selection too
+  int nblk_extra = 0;
+};
+
+// Launch shape of the FP64 per-tet kernels. A warp instruction holds an SM's
+// FP64 pipe for 16 cycles, so a mesh that fits in one warp per block is
+// spread one warp at a time over the SMs (128-thread blocks left 140 of 152
+// SMs idle on a 1,536-tet beam: gradient 69, direction 18, line search 29,
+// update 27 us). From 8 warps per SM on (m > 256 per SM) every SM is busy
+// either way and 128-thread blocks keep the partial sums few.
+inline void tet64_shape(int64_t m, int sms, int* grid, int* threads) {
+  *threads = m <= 256 * (int64_t)sms ? 32 : 128;
+  const int64_t g = (m + *threads - 1) / *threads;
+  *grid = (int)(g < 1 ? 1 : g > 8 * (int64_t)sms ? 8 * (int64_t)sms : g);
+}
+
 // Arrays the per-tet kernels read and write. FP64 path: TW = double.
 // Mixed path: TW = float for the Hessian / Woodbury quantities (Uw, y, d, gam).
 template <typename TW> struct TetArgs {
@@ -41,11 +63,13 @@ template <typename TW> struct TetArgs {
 };
 
 void launch_rhs_from_state(const TetArgs<double>& a, int grid, cudaStream_t st);
-template <typename TW> void launch_grad(const TetArgs<TW>& a, int grid, cudaStream_t st);
+// threads: 32 or 128 per block (tet64_shape)
+template <typename TW> void launch_grad(const TetArgs<TW>& a, int grid, int threads, cudaStream_t st);
 template <typename TW> void launch_syrk(const TetArgs<TW>& a, int grid, double* cpart, cudaStream_t st);
-template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, cudaStream_t st);
-template <typename TW> void launch_ls(const TetArgs<TW>& a, int grid, double rho, cudaStream_t st);
-template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, cudaStream_t st);
+template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, int threads, cudaStream_t st);
+template <typename TW> void launch_ls(const TetArgs<TW>& a, int grid, int threads, const LsSelect& sel, cudaStream_t st);
+// per-tet state and, for q += sigma dq, the vertices (3 n values of a.dq)
+template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, int threads, double* q, cudaStream_t st);
 
 // Per-vertex RHS gather: b_v = sum over incident corner slots, minus the
 // pinned-column term (mode 0, coupling solve for q) or not (mode 1, dq).
@@ -58,9 +82,6 @@ void launch_update_verts(int64_t n, const DevScalars* sc, const double* dq, doub
 void launch_nu(int64_t m, const int4* tet, const double* Dinv, const double* w, const double* x, double* nu64,
                float* nu32, cudaStream_t st);
 
-// Single-block reducers.
-void launch_reduce_grad(const double* partials, int nblk, DevScalars* sc, double* By, double* gsum,
-                        cudaStream_t st);
 // cpart: entry-major partials (kCapEntries + kK entries x nblk blocks);
 // cfull_scratch receives their sums. fp32_factor: factor and solve in FP32.
 // cadd (null, or kCapEntries + kK values) is added to the summed entries
@@ -69,8 +90,6 @@ void launch_cap_solve(const double* cpart, int nblk, const double* cfull_scratch
                       bool fp32_factor, cudaStream_t st, const double* cadd = nullptr);
 // Restart the line search: ls_fail = 0, sigma_start = sigma0.
 void launch_ls_reset(DevScalars* sc, double sigma0, cudaStream_t st);
-void launch_ls_select(const double* dir_partials, int nblk_dir, const double* ls_partials, int nblk_ls,
-                      DevScalars* sc, double sigma0, double rho, double c_armijo, cudaStream_t st);
 
 // Normaliser of the residual: ||g(F = I, q0)||^2 into out[0].
 void launch_gref(const TetArgs<double>& a, const double* q0, int grid, double* partials, double* out,
@@ -143,6 +162,27 @@ __device__ __forceinline__ void ls_select_block(const double* dir_partials, int 
   }
 }
 
+// The gradient kernels' last block to finish sums the squared gradient norm
+// (one partial per block).
+__device__ __forceinline__ void grad_finish(DevScalars* sc, const double* partials) {
+  if (!last_block(&sc->ticket[kTicketGrad])) return;
+  __shared__ double tot[1];
+  block_sum_partials<1>(partials, gridDim.x, tot);
+  if (threadIdx.x == 0) {
+    sc->gnorm2 = tot[0];
+    sc->ticket[kTicketGrad] = 0u;
+  }
+}
+
+// The line-search kernels' last block sums every block's partials and selects the step.
+__device__ __forceinline__ void ls_finish(DevScalars* sc, const double* partials, const LsSelect& sel) {
+  if (!last_block(&sc->ticket[kTicketLs])) return;
+  ls_select_block(sel.dir_partials, sel.nblk_dir, partials, gridDim.x + sel.nblk_extra, sc, sel.sigma0, sel.rho,
+                  sel.c_armijo);
+  if (threadIdx.x == 0) sc->ticket[kTicketLs] = 0u;
+}
+
+constexpr int kSyrk64Chunk = 4;       // tets per chunk of the FP64 capacitance kernels
 constexpr int kCapEntries = kK * kK;   // 48 x 48 partial capacitance
 
 // The 3 x 3 tiles of the lower triangle of the 48 x 48 symmetric product

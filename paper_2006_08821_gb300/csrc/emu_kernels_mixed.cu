@@ -160,15 +160,7 @@ __global__ void __launch_bounds__(128, 4) k_grad_m(MixArgs a) {
   double acc[1] = {(double)accf};
   block_reduce_write<1>(acc, a.partials + blockIdx.x);
   if (bad) atomicExch(&a.sc->nonfinite, 1);
-  // the last block to finish sums the squared gradient norm
-  if (last_block(&a.sc->ticket[kTicketGrad])) {
-    __shared__ double tot[1];
-    block_sum_partials<1>(a.partials, gridDim.x, tot);
-    if (threadIdx.x == 0) {
-      a.sc->gnorm2 = tot[0];
-      a.sc->ticket[kTicketGrad] = 0u;
-    }
-  }
+  grad_finish(a.sc, a.partials);
 }
 
 void launch_grad_mixed(const MixArgs& a, int grid, cudaStream_t st) { k_grad_m<<<grid, 128, 0, st>>>(a); }
@@ -582,12 +574,7 @@ __global__ void __launch_bounds__(128) k_ls_m(MixArgs a, LsSelect sel) {
 #pragma unroll
   for (int k = 0; k < kLsNV; ++k) acc[k] = (double)accf[k];
   block_reduce_write<kLsNV>(acc, a.partials + (size_t)blockIdx.x * kLsNV);
-  // the last block to finish sums every block's partials and selects the step
-  if (last_block(&a.sc->ticket[kTicketLs])) {
-    ls_select_block(sel.dir_partials, sel.nblk_dir, a.partials, gridDim.x + sel.nblk_extra, a.sc, sel.sigma0, sel.rho,
-                    sel.c_armijo);
-    if (threadIdx.x == 0) a.sc->ticket[kTicketLs] = 0u;
-  }
+  ls_finish(a.sc, a.partials, sel);
 }
 
 void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream_t st) {

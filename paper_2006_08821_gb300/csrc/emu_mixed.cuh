@@ -57,15 +57,6 @@ struct MixArgs {
 void launch_grad_mixed(const MixArgs& a, int grid, cudaStream_t st);
 void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st);
 // Line-search constants and the direction kernel's g.d partials, for the
-// Armijo selection the last block of the line-search kernel performs.
-struct LsSelect {
-  const double* dir_partials;
-  int nblk_dir;
-  double sigma0, rho, c_armijo;
-  // blocks of line-search partials written after the kernel's own (the free
-  // bones' FP64 terms, Sec. 3.3), summed by the selection too
-  int nblk_extra = 0;
-};
 // Trial energies of one pass and, in its last block, the selected step
 // (k_ls_select's work); the gradient kernel likewise leaves ||g||^2 in sc.
 void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream_t st);
