@@ -23,7 +23,7 @@
 
 namespace emu {
 namespace {
-int enqueue_grad(emu_handle* h);
+int enqueue_grad(emu_handle* h, bool split = true);
 int enqueue_direction(emu_handle* h);
 }  // namespace
 }  // namespace emu
@@ -1338,6 +1338,7 @@ struct SolveTask {
   double res = 0.0, gnorm_ref = 0.0;
   bool first_eval = true;
   bool ls_refreshed = false;  // q re-solved during the current run of rejected passes
+  bool split = true;          // q was re-solved since the displacement's float pair was formed
   bool ref_short = false;     // the last exact re-solve stopped above its tolerance
   bool ls_retried = false;    // and dq tightened after it, too
   double best_res = 1e300;    // smallest residual so far and the iteration it was seen
@@ -1362,18 +1363,19 @@ bool task_ready(const SolveTask* t) {
 
 namespace {
 // enqueue the gradient and its reduction, then wait for the scalars
-int enqueue_grad(emu_handle* h) {
+// (split: form the displacement's float pair from q first; the update kernel
+// has left it when q was only advanced by a step since)
+int enqueue_grad(emu_handle* h, bool split) {
   h->ph_begin();
   if (h->mixed) {
-    // the displacement's float pair for this iteration's per-tet kernels
-    launch_split_disp(h->n, h->q, h->Qrest, h->uh32, h->ul32, h->st);
+    if (split) launch_split_disp(h->n, h->q, h->Qrest, h->uh32, h->ul32, h->st);
     launch_grad_mixed(h->margs(), h->grid_tet4, h->st);
   } else if (h->fform) {
     launch_grad_fform(h->args<double>(), h->grid_t64, h->threads_t64, h->st);
   } else {
     launch_grad<double>(h->args<double>(), h->grid_t64, h->threads_t64, h->st);
   }
-  h->ph_end(EMU_PHASE_GRAD, h->mixed ? 2 : 1);
+  h->ph_end(EMU_PHASE_GRAD, h->mixed && split ? 2 : 1);
   if (h->nfb > 0) {  // the free bones' virtual elements (Sec. 3.3)
     h->ph_begin();
     bones_after_grad(h);
@@ -1467,41 +1469,46 @@ int enqueue_step(emu_handle* h) {
   h->ph_end(EMU_PHASE_LS, 1);
   h->ph_begin();
   if (h->mixed) {
-    launch_update_mixed(am, h->grid_tet, h->st);
+    launch_update_mixed(am, h->grid_tet, h->q, cg64(h) ? h->dq : nullptr, h->uh32, h->ul32, h->st);
     bones_update_mixed(h);
-    if (cg64(h))
-      launch_update_verts(h->n, h->sc, h->dq, h->q, h->st);
-    else
-      launch_update_verts_f(h->n, h->sc, h->dq32, h->q, h->st);
   } else {
     if (h->fform)
       launch_update_fform(a64, h->grid_tet, h->q, h->st);
     else
       launch_update_tets<double>(a64, h->grid_t64, h->threads_t64, h->q, h->st);
   }
-  h->ph_end(EMU_PHASE_UPDATE, h->mixed ? 2 : 1);
+  h->ph_end(EMU_PHASE_UPDATE, 1);
   EMU_CK(cudaGetLastError());
   return EMU_OK;
 }
 // Enqueues enqueue_step + enqueue_grad as one CUDA graph launch (captured
 // on first use and again when the dq tolerance or first trial step changes). Returns 1 when the
 // graph was launched, 0 when the caller must enqueue directly (profiling
-// on, the legacy default stream, or a capture that failed).
+// on, or a capture that failed).
 int launch_iteration_graph(emu_handle* h) {
-  if (!h->graphs_ok || h->prof_on || h->st == nullptr) return 0;
+  if (!h->graphs_ok || h->prof_on) return 0;
   if (!h->iter_exec || h->iter_exec_dq != h->dq_tol_now || h->iter_exec_sigma0 != h->sigma0_now) {
     if (h->iter_exec) cudaGraphExecDestroy(h->iter_exec);
     h->iter_exec = nullptr;
-    if (cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    // the legacy default stream cannot be captured: the nodes are recorded on
+    // a stream that exists for the capture only and launched on the handle's
+    cudaStream_t const own = h->st;
+    cudaStream_t cap = own;
+    if ((own == nullptr && cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) ||
+        cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
+      if (own == nullptr && cap) cudaStreamDestroy(cap);
       h->graphs_ok = false;
       return 0;
     }
+    h->st = cap;
     const int64_t launches0 = h->launches;
     int rc = enqueue_step(h);
-    if (!rc) rc = enqueue_grad(h);
+    if (!rc) rc = enqueue_grad(h, false);
     cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(h->st, &g);
+    const cudaError_t e = cudaStreamEndCapture(cap, &g);
+    h->st = own;
+    if (cap != own) cudaStreamDestroy(cap);
     h->iter_graph_kernels = h->launches - launches0;  // kernels of one launch
     h->launches = launches0;                          // nothing ran yet
     cudaGraphExec_t ex = nullptr;
@@ -1630,6 +1637,7 @@ int task_step(SolveTask* t) {
           rc = refresh_begin(h, h->q_tol);
           if (rc) return abort(rc);
           t->round = 0;
+          t->split = true;
           t->phase = SolveTask::REF_RES;
           break;
         }
@@ -1656,8 +1664,9 @@ int task_step(SolveTask* t) {
         break;
       }
       case SolveTask::GRAD:
-        rc = enqueue_grad(h);
+        rc = enqueue_grad(h, t->split);
         if (rc) return abort(rc);
+        t->split = false;
         t->phase = SolveTask::DECIDE;
         return wait();
       case SolveTask::DECIDE: {

@@ -40,45 +40,33 @@ void launch_rhs_from_state(const TetArgs<double>& a, int grid, cudaStream_t st) 
   k_rhs_from_state<<<grid, 256, 0, st>>>(a);
 }
 
-__global__ void __launch_bounds__(256) k_assemble(int64_t n, const int32_t* __restrict__ slot_ptr,
+// One thread per vertex and coordinate: the corner terms are added in slot
+// order, eight in flight with the next eight indices, so a vertex of 24 corners
+// costs four L2 round trips instead of a chain through every slot (425
+// vertices 12.6 us, 1,485 in FP32 8.1 us before).
+__global__ void __launch_bounds__(128) k_assemble(int64_t n, const int32_t* __restrict__ slot_ptr,
                                                   const int32_t* __restrict__ slot_idx,
                                                   const double* __restrict__ contrib, const double* __restrict__ bfix,
                                                   const uint8_t* __restrict__ is_fixed,
                                                   const double* __restrict__ qfix, int mode, double* __restrict__ b) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    double s0 = 0, s1 = 0, s2 = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = i / 3;
+    double s = 0.0;
     if (is_fixed[v]) {
-      if (mode == 0) {
-        s0 = qfix[3 * v];
-        s1 = qfix[3 * v + 1];
-        s2 = qfix[3 * v + 2];
-      }
+      if (mode == 0) s = qfix[i];
     } else {
-      const int32_t e0 = slot_ptr[v], e1 = slot_ptr[v + 1];
-      for (int32_t e = e0; e < e1; ++e) {
-        const int64_t sl = slot_idx[e];
-        s0 += contrib[3 * sl];
-        s1 += contrib[3 * sl + 1];
-        s2 += contrib[3 * sl + 2];
-      }
-      if (mode == 0) {
-        s0 -= bfix[3 * v];
-        s1 -= bfix[3 * v + 1];
-        s2 -= bfix[3 * v + 2];
-      }
+      s = gather_corners(slot_idx, slot_ptr[v], slot_ptr[v + 1], contrib + (i - 3 * v));
+      if (mode == 0) s -= bfix[i];
     }
-    b[3 * v] = s0;
-    b[3 * v + 1] = s1;
-    b[3 * v + 2] = s2;
+    b[i] = s;
   }
 }
 
 void launch_assemble(int64_t n, const int32_t* slot_ptr, const int32_t* slot_idx, const double* contrib,
                      const double* bfix, const uint8_t* is_fixed, const double* qfix, int mode, double* b,
                      cudaStream_t st) {
-  int grid = (int)((n + 255) / 256);
-  if (grid < 1) grid = 1;
-  k_assemble<<<grid, 256, 0, st>>>(n, slot_ptr, slot_idx, contrib, bfix, is_fixed, qfix, mode, b);
+  const int64_t grid = (3 * n + 127) / 128;
+  k_assemble<<<(int)(grid < 1 ? 1 : grid), 128, 0, st>>>(n, slot_ptr, slot_idx, contrib, bfix, is_fixed, qfix, mode, b);
 }
 
 // ------------------------------------------------------------ gradient ----
@@ -256,21 +244,24 @@ template <typename TW> void launch_syrk(const TetArgs<TW>& a, int grid, double* 
 }
 
 // ------------------------------------------- capacitance sum and solve ----
-// 1 / d by Newton's iteration from a hardware estimate (its error is at most
-// an ulp; one step leaves rounding), without a division's range handling.
-__device__ __forceinline__ float pivot_inverse(float d) {
-  if (!(d > 1e-30f && d < 1e30f)) return 1.f / d;
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-  return fmaf(r, fmaf(-d, r, 1.f), r);
-}
-// Newton's iteration for 1 / d from an FP32 start (relative error 1e-7, 1e-14,
-// then rounding): six dependent operations instead of a division's sequence.
+__device__ __forceinline__ float pivot_inverse(float d) { return __frcp_rn(d); }
+// 1 / d in FP64 by Newton's iteration: the hardware estimate is good to 2^-20
+// or so, and one cubic step (error e -> e^3) leaves rounding. Three FP64 instructions; the range
+// test is on the exponent's integer bits (an FP64 comparison costs a warp as
+// much as a multiplication).
 __device__ __forceinline__ double pivot_inverse(double d) {
-  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
-  double r = (double)(1.f / (float)d);
-  r = fma(r, fma(-d, r, 1.0), r);
-  return fma(r, fma(-d, r, 1.0), r);
+  const int hi = __double2hiint(d);
+  if (!(hi > 0x01000000 && hi < 0x7e000000)) return 1.0 / d;  // outside 2^-1007 .. 2^993
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ bool positive(float x) { return x > 0.f; }
+// x > 0 (false for NaN) on the bits
+__device__ __forceinline__ bool positive(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
 constexpr int kCapLow = kK * (kK + 1) / 2;        // entries of the lower triangle
@@ -286,8 +277,8 @@ constexpr int kCapOwn = (kCapSums + 255) / 256;   // entries a thread of the sol
 // Latency decides here: one block, 48 dependent pivots. Each of the 256
 // threads owns up to five entries of the lower triangle in registers, with
 // B y as row 48, so the forward substitution is part of the factorisation.
-// Per panel of four columns the owners hand the panel to one warp, which
-// factors it with its rows in registers (shuffles instead of barriers), and
+// Per panel of four columns the owners hand the panel to two warps, which
+// factor it with their rows in registers (shuffles instead of barriers), and
 // every thread then applies the four rank-1 updates to its entries: two block
 // barriers per four columns, and the work of the trailing triangle only. The
 // entries are numbered from the last column backwards, so the trailing
@@ -318,92 +309,145 @@ __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, i
       if (lane == 0) __stcg(cfull + src, cadd ? x + cadd[src] : x);
     }
   }
-  if (!last_block(&sc->ticket[kTicketCap])) return;
-  __shared__ T sL[kK + 1][kK + 1];      // finished columns of L; row 48: D^-1 L^-1 (B y)
-  __shared__ T sP[kCapNB][kK + 1];      // the panel's columns
-  __shared__ T sW[kCapNB][kK + 1];      // L D of the panel
-  __shared__ int s_ok;
   // entry t: column 48 - a and row 48 - b with 0 <= b <= a, t = a (a + 1) / 2 + b (a = 0 is unused)
   int row[kCapOwn], col[kCapOwn];
-  T val[kCapOwn];
 #pragma unroll
   for (int s = 0; s < kCapOwn; ++s) {
     const int t = 1 + tid + 256 * s;
     int a = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-    while ((a + 1) * (a + 2) / 2 <= t) ++a;
-    while (a * (a + 1) / 2 > t) --a;
-    col[s] = kK - a;
+    if ((a + 1) * (a + 2) / 2 <= t) ++a;
+    if (a * (a + 1) / 2 > t) --a;
+    col[s] = t <= kCapSums ? kK - a : -1;
     row[s] = kK - (t - a * (a + 1) / 2);
-    val[s] = T(0);
-    if (t <= kCapSums) {
-      const double diag = __ldcg(cfull + col[s] * kK + col[s]);
-      const double v = row[s] < kK ? __ldcg(cfull + row[s] * kK + col[s]) : __ldcg(cfull + kCapEntries + col[s]);
-      val[s] = (T)v;
-      // unused modes (k_modes < 48) have zero rows: identity rows with a zero right-hand side
-      if (diag == 0.0) val[s] = row[s] == col[s] ? T(1) : row[s] == kK ? T(0) : val[s];
-    } else {
-      col[s] = -1;
-    }
+  }
+  if (!last_block(&sc->ticket[kTicketCap])) return;
+  // In FP64 B y is row 48 of the factorisation, which leaves D^-1 L^-1 (B y)
+  // there. In FP32 the third warp substitutes with 1 / sqrt(d) scaling while
+  // the others update (the mixed path's rounding, and so its iterates, are
+  // those of a plain column-by-column factorisation).
+  constexpr bool kRowB = sizeof(T) == 8;
+  __shared__ T sL[kK + 1][kK + 1];      // finished columns, scaled by 1 / d (FP32: unscaled)
+  __shared__ T sP[kCapNB][kK + 1];      // the panel's columns
+  __shared__ T sW[2][kCapNB][kK + 1];   // the finished columns of this and the last panel, unscaled
+  __shared__ T sS[kCapNB][kK + 1];      // and scaled by 1 / d
+  __shared__ T sR[kK];                  // FP32: 1 / sqrt(d)
+  __shared__ int s_ok;
+  T val[kCapOwn];
+#pragma unroll
+  for (int s = 0; s < kCapOwn; ++s) {
+    const int c = col[s] < 0 ? 0 : col[s];
+    const double diag = __ldcg(cfull + c * kK + c);
+    const double v = row[s] < kK ? __ldcg(cfull + row[s] * kK + c) : __ldcg(cfull + kCapEntries + c);
+    val[s] = (T)v;
+    // unused modes (k_modes < 48) have zero rows: identity rows with a zero right-hand side
+    if (diag == 0.0) val[s] = row[s] == c ? T(1) : row[s] == kK ? T(0) : val[s];
   }
   if (tid == 0) s_ok = 1;
-  for (int p0 = 0; p0 < kK; p0 += kCapNB) {
+  T x0 = T(0), x1 = T(0);  // FP32: right-hand side rows lane and 32 + lane of the third warp
+  const bool has1 = lane + 32 < kK;
+  if (!kRowB && tid >= 64 && tid < 96) {
+    if (__ldcg(cfull + lane * kK + lane) != 0.0) x0 = (T)__ldcg(cfull + kCapEntries + lane);
+    if (has1 && __ldcg(cfull + (lane + 32) * kK + lane + 32) != 0.0) x1 = (T)__ldcg(cfull + kCapEntries + lane + 32);
+  }
+  // L y = b, y_j = x_j / L_jj with L_ij = C_ij / sqrt(d_j) (FP32, the third
+  // warp), for the columns of the panel at p0; the four roots in four lanes
+  auto substitute = [&](int p0, const T (*W)[kK + 1]) {
+    const T d4 = W[lane & (kCapNB - 1)][p0 + (lane & (kCapNB - 1))];
+    const T ri4 = positive(d4) ? T(1) / sqrt(d4) : T(1);
+    if (lane < kCapNB) sR[p0 + lane] = ri4;
+#pragma unroll
+    for (int p = 0; p < kCapNB; ++p) {
+      const int j = p0 + p;
+      const T ri = __shfl_sync(0xffffffffu, ri4, p);
+      const T yj = __shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31) * ri;
+      const T f = ri * yj;
+      if (lane == (j & 31)) {
+        if (j < 32) x0 = yj; else x1 = yj;
+      }
+      if (lane > j) x0 -= W[p][lane] * f;
+      if (has1 && lane + 32 > j) x1 -= W[p][lane + 32] * f;
+    }
+  };
+  for (int p0 = 0, buf = 0; p0 < kK; p0 += kCapNB, buf ^= 1) {
 #pragma unroll
     for (int s = 0; s < kCapOwn; ++s)
       if (col[s] >= p0 && col[s] < p0 + kCapNB) sP[col[s] - p0][row[s]] = val[s];
     __syncthreads();
-    if (tid < 32) {
-      // rows p0 + lane and p0 + 32 + lane of the panel
-      const int ra = p0 + lane, rb = ra + 32;
-      T va[kCapNB], vb[kCapNB];
+    if (tid < 64) {
+      // row of this lane: warp 0 takes p0 .. p0 + 31; warp 1 copies of the
+      // four pivot rows in its first lanes, then p0 + 32 ..
+      const bool copy = tid >= 32 && lane < kCapNB;
+      const int r = tid < 32 || copy ? p0 + lane : p0 + 32 - kCapNB + lane;
+      const bool on = r <= kK && !copy;
+      T v[kCapNB];
 #pragma unroll
-      for (int q = 0; q < kCapNB; ++q) {
-        va[q] = (ra <= kK && ra >= p0 + q) ? sP[q][ra] : T(0);
-        vb[q] = rb <= kK ? sP[q][rb] : T(0);
-      }
+      for (int q = 0; q < kCapNB; ++q) v[q] = r <= kK && r >= p0 + q ? sP[q][r] : T(0);
 #pragma unroll
       for (int p = 0; p < kCapNB; ++p) {
-        T d = __shfl_sync(0xffffffffu, va[p], p);
-        if (!(d > T(0))) {  // not positive definite: recorded, z = 0 below
+        T d = __shfl_sync(0xffffffffu, v[p], p);
+        if (!positive(d)) {  // not positive definite: recorded, z = 0 below
           d = T(1);
           s_ok = 0;
         }
-        const T ri = pivot_inverse(d);
-        if (ra <= kK) sW[p][ra] = va[p];
-        if (rb <= kK) sW[p][rb] = vb[p];
-#pragma unroll
-        for (int q = p + 1; q < kCapNB; ++q) {
-          const T l = __shfl_sync(0xffffffffu, va[p], q) * ri;
-          va[q] -= va[p] * l;
-          vb[q] -= vb[p] * l;
+        const T l = v[p] * pivot_inverse(d);
+        if (on) {
+          sW[buf][p][r] = v[p];
+          sS[p][r] = l;
+          sL[r][p0 + p] = kRowB ? l : v[p];
         }
-        if (ra <= kK) sL[ra][p0 + p] = va[p] * ri;
-        if (rb <= kK) sL[rb][p0 + p] = vb[p] * ri;
+#pragma unroll
+        for (int q = p + 1; q < kCapNB; ++q) v[q] -= l * __shfl_sync(0xffffffffu, v[p], q);
       }
+    } else if (!kRowB && tid < 96 && p0 > 0) {
+      substitute(p0 - kCapNB, sW[buf ^ 1]);  // one panel behind, while this one is factored
     }
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < kCapOwn; ++s)
       if (col[s] >= p0 + kCapNB) {
 #pragma unroll
-        for (int q = 0; q < kCapNB; ++q) val[s] -= sW[q][row[s]] * sL[col[s]][p0 + q];
+        for (int q = 0; q < kCapNB; ++q) val[s] -= sS[q][row[s]] * sW[buf][q][col[s]];
       }
   }
-  if (tid < 32) {  // L^T z = y
-    const bool has1 = lane + 32 < kK;
-    T x0 = sL[kK][lane], x1 = has1 ? sL[kK][lane + 32] : T(0);
+  if (tid < 64 || tid >= 96) return;
+  if constexpr (kRowB) {  // L^T z = y with L unit lower triangular
+    x0 = sL[kK][lane];
+    if (has1) x1 = sL[kK][lane + 32];
 #pragma unroll 4
-    for (int j = kK - 1; j > 0; --j) {
-      const T zj = __shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31);
+    for (int j = kK - 1; j >= 32; --j) {
+      const T zj = __shfl_sync(0xffffffffu, x1, j & 31);
+      x0 -= sL[j][lane] * zj;
+      if (lane + 32 < j) x1 -= sL[j][lane + 32] * zj;
+    }
+#pragma unroll 4
+    for (int j = 31; j > 0; --j) {
+      const T zj = __shfl_sync(0xffffffffu, x0, j);
       if (lane < j) x0 -= sL[j][lane] * zj;
-      if (has1 && lane + 32 < j) x1 -= sL[j][lane + 32] * zj;
     }
-    const int ok = s_ok;
-    z[lane] = ok ? (double)x0 : 0.0;
-    if (has1) z[lane + 32] = ok ? (double)x1 : 0.0;
-    if (lane == 0) {
-      sc->cap_ok = ok ? 1.0 : 0.0;
-      sc->ticket[kTicketCap] = 0u;
+  } else {  // z_j = x_j / L_jj, then x_i -= L_ji z_j for i < j
+    substitute(kK - kCapNB, sW[(kK / kCapNB - 1) & 1]);
+    __syncwarp();
+    const T r0 = sR[lane], r1 = has1 ? sR[lane + 32] : T(0);
+#pragma unroll 4
+    for (int j = kK - 1; j >= 32; --j) {
+      const T zj = __shfl_sync(0xffffffffu, x1, j & 31) * sR[j];
+      if (lane == (j & 31)) x1 = zj;
+      x0 -= sL[j][lane] * r0 * zj;
+      if (lane + 32 < j) x1 -= sL[j][lane + 32] * r1 * zj;
     }
+#pragma unroll 4
+    for (int j = 31; j >= 0; --j) {
+      const T zj = __shfl_sync(0xffffffffu, x0, j) * sR[j];
+      if (lane == j) x0 = zj;
+      if (lane < j) x0 -= sL[j][lane] * r0 * zj;
+    }
+  }
+  const int ok = s_ok;
+  z[lane] = ok ? (double)x0 : 0.0;
+  if (has1) z[lane + 32] = ok ? (double)x1 : 0.0;
+  if (lane == 0) {
+    sc->cap_ok = ok ? 1.0 : 0.0;
+    sc->ticket[kTicketCap] = 0u;
   }
 }
 
@@ -619,20 +663,6 @@ __global__ void __launch_bounds__(128) k_update_tets(TetArgs<TW> a, double* __re
 
 template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, int threads, double* q, cudaStream_t st) {
   k_update_tets<TW><<<grid, threads, 0, st>>>(a, q);
-}
-
-__global__ void __launch_bounds__(256) k_update_verts(int64_t n3, const DevScalars* sc, const double* dq, double* q) {
-  const double sig = sc->sigma;
-  if (sig == 0.0) return;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n3; k += (int64_t)gridDim.x * blockDim.x)
-    q[k] += sig * dq[k];
-}
-
-void launch_update_verts(int64_t n, const DevScalars* sc, const double* dq, double* q, cudaStream_t st) {
-  int64_t n3 = 3 * n;
-  int grid = (int)((n3 + 255) / 256);
-  if (grid < 1) grid = 1;
-  k_update_verts<<<grid, 256, 0, st>>>(n3, sc, dq, q);
 }
 
 // ------------------------------------------------------------ normaliser --

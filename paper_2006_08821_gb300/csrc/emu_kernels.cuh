@@ -76,7 +76,6 @@ template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, i
 void launch_assemble(int64_t n, const int32_t* slot_ptr, const int32_t* slot_idx, const double* contrib,
                      const double* bfix, const uint8_t* is_fixed, const double* qfix, int mode, double* b,
                      cudaStream_t st);
-void launch_update_verts(int64_t n, const DevScalars* sc, const double* dq, double* q, cudaStream_t st);
 // Generalized external force of Sec. 3.4: nu_i = w_i G_i x (x = K^-1 f, 3n),
 // written component-major to nu64 (9m) and, when non-null, nu32.
 void launch_nu(int64_t m, const int4* tet, const double* Dinv, const double* w, const double* x, double* nu64,
@@ -160,6 +159,28 @@ __device__ __forceinline__ void ls_select_block(const double* dir_partials, int 
     sc->ls_trials += kLsTrials;
     sc->ls_fail += 1;
   }
+}
+
+// Sum of contrib[3 slot_idx[e]] over e0 <= e < e1 in that order.
+template <typename T>
+__device__ __forceinline__ T gather_corners(const int32_t* __restrict__ slot_idx, int32_t e0, int32_t e1,
+                                            const T* __restrict__ contrib) {
+  constexpr int W = 8;
+  T s = T(0);
+  int32_t idx[W];
+#pragma unroll
+  for (int t = 0; t < W; ++t) idx[t] = e0 + t < e1 ? __ldg(slot_idx + e0 + t) : 0;
+  for (int32_t e = e0; e < e1; e += W) {
+    T x[W];
+#pragma unroll
+    for (int t = 0; t < W; ++t) x[t] = e + t < e1 ? contrib[3 * (int64_t)idx[t]] : T(0);
+#pragma unroll
+    for (int t = 0; t < W; ++t) idx[t] = e + W + t < e1 ? __ldg(slot_idx + e + W + t) : 0;
+#pragma unroll
+    for (int t = 0; t < W; ++t)
+      if (e + t < e1) s += x[t];
+  }
+  return s;
 }
 
 // The gradient kernels' last block to finish sums the squared gradient norm

@@ -584,11 +584,24 @@ void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream
 // ------------------------------------------------------------ update ------
 // F' = R (S + s R^T d) = R (I + Y), Y = E + s R^T d; I + Y = Rx (I + E'):
 // q' = q Rx, E' from the near-identity polar factor.
-__global__ void __launch_bounds__(128) k_update_m(MixArgs a) {
+// The vertices ride along: q += sigma dq (dq64 where the coupling solve runs in
+// FP64, else the FP32 dq) and the displacement's float pair that the next
+// gradient reads (one launch instead of three; a rejected step, sigma = 0,
+// changes none of them).
+__global__ void __launch_bounds__(128) k_update_m(MixArgs a, double* __restrict__ q, const double* __restrict__ dq64,
+                                                  float* __restrict__ uh, float* __restrict__ ul) {
   const double sigd = a.sc->sigma;
   if (sigd == 0.0) return;
   const float sig = (float)sigd;
   const int64_t m = a.m;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < 3 * a.n; k += (int64_t)gridDim.x * blockDim.x) {
+    const double qn = q[k] + sigd * (dq64 ? dq64[k] : (double)a.dq[k]);
+    const double u = qn - a.Q[k];
+    const float hi = (float)u;
+    q[k] = qn;
+    uh[k] = hi;
+    ul[k] = (float)(u - (double)hi);
+  }
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     if (a.tkind && a.tkind[i] != kTetDeformable) continue;  // bones: FP64 state of their own
     float R[9], e6[6], d[9], Rtd[9], Y[9];
@@ -609,13 +622,9 @@ __global__ void __launch_bounds__(128) k_update_m(MixArgs a) {
   }
 }
 
-void launch_update_mixed(const MixArgs& a, int grid, cudaStream_t st) { k_update_m<<<grid, 128, 0, st>>>(a); }
-
-__global__ void __launch_bounds__(256) k_update_verts_f(int64_t n3, const DevScalars* sc, const float* dq, double* q) {
-  const double sig = sc->sigma;
-  if (sig == 0.0) return;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n3; k += (int64_t)gridDim.x * blockDim.x)
-    q[k] += sig * (double)dq[k];
+void launch_update_mixed(const MixArgs& a, int grid, double* q, const double* dq64, float* uh, float* ul,
+                         cudaStream_t st) {
+  k_update_m<<<grid, 128, 0, st>>>(a, q, dq64, uh, ul);
 }
 
 __global__ void __launch_bounds__(256) k_split_disp(int64_t n3, const double* __restrict__ q, const double* __restrict__ Q,
@@ -633,13 +642,6 @@ void launch_split_disp(int64_t n, const double* q, const double* Q, float* uh, f
   int grid = (int)((n3 + 255) / 256);
   if (grid < 1) grid = 1;
   k_split_disp<<<grid, 256, 0, st>>>(n3, q, Q, uh, ul);
-}
-
-void launch_update_verts_f(int64_t n, const DevScalars* sc, const float* dq, double* q, cudaStream_t st) {
-  const int64_t n3 = 3 * n;
-  int grid = (int)((n3 + 255) / 256);
-  if (grid < 1) grid = 1;
-  k_update_verts_f<<<grid, 256, 0, st>>>(n3, sc, dq, q);
 }
 
 // ------------------------------------------------------- coupling RHS ----
@@ -704,32 +706,21 @@ __global__ void __launch_bounds__(256) k_rhs_state_m(MixArgs a) {
 
 void launch_rhs_state_mixed(const MixArgs& a, int grid, cudaStream_t st) { k_rhs_state_m<<<grid, 256, 0, st>>>(a); }
 
-__global__ void __launch_bounds__(256) k_assemble_f(int64_t n, const int32_t* __restrict__ slot_ptr,
+// b of the dq solve from the FP32 corner terms, as k_assemble
+__global__ void __launch_bounds__(128) k_assemble_f(int64_t n, const int32_t* __restrict__ slot_ptr,
                                                     const int32_t* __restrict__ slot_idx,
                                                     const float* __restrict__ contrib,
                                                     const uint8_t* __restrict__ is_fixed, float* __restrict__ b) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    if (!is_fixed[v]) {
-      const int32_t e0 = slot_ptr[v], e1 = slot_ptr[v + 1];
-      for (int32_t e = e0; e < e1; ++e) {
-        const int64_t sl = slot_idx[e];
-        s0 += contrib[3 * sl];
-        s1 += contrib[3 * sl + 1];
-        s2 += contrib[3 * sl + 2];
-      }
-    }
-    b[3 * v] = s0;
-    b[3 * v + 1] = s1;
-    b[3 * v + 2] = s2;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = i / 3;
+    b[i] = is_fixed[v] ? 0.f : gather_corners(slot_idx, slot_ptr[v], slot_ptr[v + 1], contrib + (i - 3 * v));
   }
 }
 
 void launch_assemble_f(int64_t n, const int32_t* slot_ptr, const int32_t* slot_idx, const float* contrib,
                        const uint8_t* is_fixed, float* b, cudaStream_t st) {
-  int grid = (int)((n + 255) / 256);
-  if (grid < 1) grid = 1;
-  k_assemble_f<<<grid, 256, 0, st>>>(n, slot_ptr, slot_idx, contrib, is_fixed, b);
+  const int64_t grid = (3 * n + 127) / 128;
+  k_assemble_f<<<(int)(grid < 1 ? 1 : grid), 128, 0, st>>>(n, slot_ptr, slot_idx, contrib, is_fixed, b);
 }
 
 // ------------------------------------------------------------ conversion --

@@ -60,7 +60,8 @@ void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st);
 // Trial energies of one pass and, in its last block, the selected step
 // (k_ls_select's work); the gradient kernel likewise leaves ||g||^2 in sc.
 void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream_t st);
-void launch_update_mixed(const MixArgs& a, int grid, cudaStream_t st);
+void launch_update_mixed(const MixArgs& a, int grid, double* q, const double* dq64, float* uh, float* ul,
+                         cudaStream_t st);
 void launch_rhs_state_mixed(const MixArgs& a, int grid, cudaStream_t st);
 // Capacitance partials C and B y on TF32 tensor cores (mma.sync), grid
 // blocks striding over 32-tet chunks; cpart is entry-major (entry * grid + block).
@@ -69,7 +70,6 @@ void launch_syrk_tc(const MixArgs& a, int grid, double* cpart, cudaStream_t st);
 constexpr int kTcBlocksPerSM = 2;
 // Per-device kernel attributes of the TC SYRK (before its first launch).
 cudaError_t prepare_syrk_tc();
-void launch_update_verts_f(int64_t n, const DevScalars* sc, const float* dq, double* q, cudaStream_t st);
 // uh + ul = q - Q: hi = the FP32 rounding of the FP64 difference, lo = the
 // FP32 rounding of what hi leaves over.
 void launch_split_disp(int64_t n, const double* q, const double* Q, float* uh, float* ul, cudaStream_t st);

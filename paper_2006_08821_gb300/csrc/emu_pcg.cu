@@ -504,6 +504,10 @@ template <typename T> cudaError_t launch_pcg(int nrhs, const PcgArgsT<T>& args, 
     int g64 = 0, rows = 0;
     if (nrhs == 3 && (!args.phi || args.phit) && pcg64_shape(args.n, device_sms(), &g64, &rows))
       return launch_pcg64(args, g64, rows, st);
+    if (nrhs == 16) {
+      const int columns = pcg16_columns(args.n, grid, device_sms());
+      if (columns > 0) return launch_pcg16(args, grid, columns, st);
+    }
   }
   cudaError_t e = cudaMemsetAsync(args.bar, 0, sizeof(GridBarrier), st);
   if (e != cudaSuccess) return e;

@@ -62,6 +62,12 @@ int pcg_max_grid(int nrhs, int64_t n);
 // vector (3 n); r, w, p and s are unused.
 bool pcg64_shape(int64_t n, int sms, int* grid, int* rows);
 cudaError_t launch_pcg64(const PcgArgsT<double>& args, int grid, int rows, cudaStream_t st);
+// Sixteen columns without a coarse space, a block per 128 rows and few columns
+// (launch_pcg<double> takes it when pcg16_columns is not 0); ``grid``
+// is the generic kernel's. args.u holds the exchanged vectors, args.partials
+// 64 doubles per generic block and 16 ints.
+int pcg16_columns(int64_t n, int grid, int sms);
+cudaError_t launch_pcg16(const PcgArgsT<double>& args, int grid, int columns, cudaStream_t st);
 int device_sms();  // multiprocessors of the current device
 // phit of a coarse basis phi (n x 16) and T (16 x 16, row-major, device)
 cudaError_t launch_phit(int64_t n, const double* phi, const double* T, double* out, cudaStream_t st);

@@ -34,8 +34,13 @@ namespace {
 constexpr int NT = kPcg32Threads;  // threads per block
 constexpr int NR = 3;    // right-hand sides (x, y, z)
 constexpr int kGather = 16;  // entries of a matrix row gathered at once
-constexpr int kGatherPart = 8;  // the same for the pruned, partitioned system
-constexpr int kLocUnroll = 8;   // local-table entries of a row read at once
+// Entries gathered at once, from the pruned system and from the local table:
+// 8 where the local rows hold at most 8 (a regular grid's pruned rows hold 7),
+// 16 for the rows of an irregular mesh (about 14), whose entries beyond the
+// eighth used to run one dependent load at a time (59,840 tets: 9,400 against
+// 4,300 cycles for the local products and 4,000 against 2,600 for the SpMV of
+// a CG iteration).
+constexpr int kWideRows = 16, kNarrowRows = 8;
 constexpr int kMaxGridStrides = 8;  // grid_sum_f handles up to 256 blocks
 // words of Pcg32Work::sync, one 128-byte line apart
 constexpr int kSyncCount = 0, kSyncDone = 32, kSyncErr = 64;
@@ -58,6 +63,7 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 // error word, every other waiter sees it, and all blocks leave.
 __device__ __forceinline__ bool gbar(const Pcg32Work& wk, unsigned& epoch, int* s_flag, unsigned long long wait_ns) {
   __syncthreads();
+  if (gridDim.x == 1) return true;  // one block: its own barrier is all there is
   epoch += 1u;
   if (threadIdx.x == 0) {
     red_release_add(wk.sync + kSyncCount, 1u);
@@ -181,6 +187,7 @@ __device__ __forceinline__ void grid_sum_f(const float* __restrict__ part, int n
   float t[P];
 #pragma unroll
   for (int j = 0; j < P; ++j) t[j] = 0.f;
+  if (G == 1) return;  // out still holds this block's sums
 #pragma unroll
   for (int s = 0; s < kMaxGridStrides; ++s) {
     const int b = lane + 32 * s;
@@ -201,89 +208,67 @@ __device__ __forceinline__ void grid_sum_f(const float* __restrict__ part, int n
   __syncthreads();
 }
 
-// y = A z for the rows a thread owns (g0 + k stride, k < RPT), z read as
-// float4 per vertex (the neighbours' values). The first kGather entries of a
-// row are gathered at once, so a row costs one L2 round trip (a vertex of a
-// tetrahedral grid has at most 14 neighbours); longer rows finish in a plain
-// loop.
-template <int RPT>
-__device__ __forceinline__ void spmv_rows(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                          const float* __restrict__ val, const bool (&own)[RPT], int64_t g0,
-                                          int64_t stride, const float4* __restrict__ z, float (&y)[RPT][NR]) {
-#pragma unroll
-  for (int k = 0; k < RPT; ++k) {
-    y[k][0] = y[k][1] = y[k][2] = 0.f;
-    if (!own[k]) continue;
-    const int64_t v = g0 + k * stride;
-    const int32_t e0 = __ldg(rowptr + v), e1 = __ldg(rowptr + v + 1);
-    const int cnt = e1 - e0;
-    float4 z4[kGather];
-    float a4[kGather];
-#pragma unroll
-    for (int t = 0; t < kGather; ++t) {
-      a4[t] = 0.f;
-      z4[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (t < cnt) {
-        a4[t] = __ldg(val + e0 + t);
-        z4[t] = __ldcg(z + __ldg(col + e0 + t));
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < kGather; ++t) {
-      y[k][0] += a4[t] * z4[t].x;
-      y[k][1] += a4[t] * z4[t].y;
-      y[k][2] += a4[t] * z4[t].z;
-    }
-    for (int32_t e = e0 + kGather; e < e1; ++e) {
-      const float av = __ldg(val + e);
-      const float4 zz = __ldcg(z + __ldg(col + e));
-      y[k][0] += av * zz.x;
-      y[k][1] += av * zz.y;
-      y[k][2] += av * zz.z;
-    }
-  }
-}
+// The rows vr[k] of a partitioned system (or of the whole one), and the same
+// product with their first GW entries gathered at once. With HOLD those
+// entries stay in registers for the whole launch: every grid barrier ends in
+// an acquire, which empties L1, so rereading them cost two L2 round trips
+// before the gather itself could start (2,000 of 14,500 cycles of a CG
+// iteration on the 6,080-tet unit, 1,100 with the entries held).
+template <int RPT, int GW, bool HOLD>
+struct MatRows {
+  const int32_t* rowptr;
+  const int32_t* col;
+  const float* val;
+  int32_t e0[RPT] = {}, cnt[RPT] = {};
+  int32_t c[HOLD ? RPT : 1][GW];
+  float a[HOLD ? RPT : 1][GW];
 
-// The same product for the rows vr[k] of a partitioned system, GW entries
-// gathered at once (the pruned rows of a tetrahedral grid hold about 7).
-template <int RPT, int GW>
-__device__ __forceinline__ void spmv_rows_v(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                            const float* __restrict__ val, const bool (&own)[RPT],
-                                            const int64_t (&vr)[RPT], const float4* __restrict__ z,
-                                            float (&y)[RPT][NR]) {
+  __device__ __forceinline__ void load(const bool (&own)[RPT], const int64_t (&vr)[RPT]) {
 #pragma unroll
-  for (int k = 0; k < RPT; ++k) {
-    y[k][0] = y[k][1] = y[k][2] = 0.f;
-    if (!own[k]) continue;
-    const int64_t v = vr[k];
-    const int32_t e0 = __ldg(rowptr + v), e1 = __ldg(rowptr + v + 1);
-    const int cnt = e1 - e0;
-    float4 z4[GW];
-    float a4[GW];
+    for (int k = 0; k < RPT; ++k) {
+      e0[k] = own[k] ? __ldg(rowptr + vr[k]) : 0;
+      cnt[k] = own[k] ? __ldg(rowptr + vr[k] + 1) - e0[k] : 0;
+      if constexpr (HOLD)
 #pragma unroll
-    for (int t = 0; t < GW; ++t) {
-      a4[t] = 0.f;
-      z4[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (t < cnt) {
-        a4[t] = __ldg(val + e0 + t);
-        z4[t] = __ldcg(z + __ldg(col + e0 + t));
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < GW; ++t) {
-      y[k][0] += a4[t] * z4[t].x;
-      y[k][1] += a4[t] * z4[t].y;
-      y[k][2] += a4[t] * z4[t].z;
-    }
-    for (int32_t e = e0 + GW; e < e1; ++e) {
-      const float av = __ldg(val + e);
-      const float4 zz = __ldcg(z + __ldg(col + e));
-      y[k][0] += av * zz.x;
-      y[k][1] += av * zz.y;
-      y[k][2] += av * zz.z;
+        for (int t = 0; t < GW; ++t) {
+          c[k][t] = t < cnt[k] ? __ldg(col + e0[k] + t) : 0;
+          a[k][t] = t < cnt[k] ? __ldg(val + e0[k] + t) : 0.f;
+        }
     }
   }
-}
+
+  // y = A z, z read as float4 per row
+  __device__ __forceinline__ void mul(const float4* __restrict__ z, float (&y)[RPT][NR]) const {
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+      float4 z4[GW];
+      float a4[GW];
+#pragma unroll
+      for (int t = 0; t < GW; ++t) {
+        a4[t] = 0.f;
+        z4[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t < cnt[k]) {
+          a4[t] = HOLD ? a[HOLD ? k : 0][t] : __ldg(val + e0[k] + t);
+          z4[t] = __ldcg(z + (HOLD ? c[HOLD ? k : 0][t] : __ldg(col + e0[k] + t)));
+        }
+      }
+      y[k][0] = y[k][1] = y[k][2] = 0.f;
+#pragma unroll
+      for (int t = 0; t < GW; ++t) {
+        y[k][0] += a4[t] * z4[t].x;
+        y[k][1] += a4[t] * z4[t].y;
+        y[k][2] += a4[t] * z4[t].z;
+      }
+      for (int32_t e = GW; e < cnt[k]; ++e) {
+        const float av = __ldg(val + e0[k] + e);
+        const float4 zz = __ldcg(z + __ldg(col + e0[k] + e));
+        y[k][0] += av * zz.x;
+        y[k][1] += av * zz.y;
+        y[k][2] += av * zz.z;
+      }
+    }
+  }
+};
 
 // loc[m NR + j] += Phi[v][m] y[k][j] over the owned rows; the coarse rows of
 // a thread live in shared memory, float4 q of row k at sPhi[(q RPT + k) NT + tid]
@@ -327,7 +312,8 @@ __device__ __forceinline__ void coarse_solve4(const float* s_Einv, const float* 
 // and a bfloat16 weight (D^-1 y when the degree is 1). Every thread of the
 // block calls apply (it holds block barriers); the two product buffers
 // alternate, so one barrier per product suffices.
-template <int RPT>
+// With HOLD a thread's first LU table words stay in registers.
+template <int RPT, int LU, bool HOLD>
 struct LocalPrec {
   float4* buf;            // 2 RPT NT float4 of shared memory
   const uint32_t* table;  // RPT lw NT words of shared memory
@@ -337,6 +323,18 @@ struct LocalPrec {
   int lw;                 // 0: Jacobi only
   int degree;
   int pb;
+  uint32_t held[HOLD ? RPT : 1][LU];
+
+  __device__ __forceinline__ void load(const uint32_t* __restrict__ src) {  // src: this block's words
+    if constexpr (HOLD)
+#pragma unroll
+      for (int k = 0; k < RPT; ++k)
+#pragma unroll
+        for (int e = 0; e < LU; ++e) held[k][e] = e < lw ? __ldg(src + ((size_t)k * lw + e) * NT + threadIdx.x) : 0u;
+    // the words that are read from shared memory
+    if (!HOLD || lw > LU)
+      for (int e = threadIdx.x; e < RPT * lw * NT; e += NT) const_cast<uint32_t*>(table)[e] = __ldg(src + e);
+  }
 
   // t = O y on the block's rows, O the off-diagonal part of A_b
   __device__ __forceinline__ void off(const bool (&own)[RPT], const float (&y)[RPT][NR], float (&t)[RPT][NR]) {
@@ -350,21 +348,21 @@ struct LocalPrec {
     for (int k = 0; k < RPT; ++k) {
       float t0 = 0.f, t1 = 0.f, t2 = 0.f;
       const uint32_t* le = table + (size_t)k * lw * NT + threadIdx.x;
-      // the first kLocUnroll entries at once (all loads in flight), the rest in a loop
-      uint32_t wd[kLocUnroll];
+      // the first LU entries at once (all loads in flight), the rest in a loop
+      uint32_t wd[LU];
 #pragma unroll
-      for (int e = 0; e < kLocUnroll; ++e) wd[e] = e < lw ? le[e * NT] : 0u;
-      float4 yv[kLocUnroll];
+      for (int e = 0; e < LU; ++e) wd[e] = HOLD ? held[HOLD ? k : 0][e] : e < lw ? le[e * NT] : 0u;
+      float4 yv[LU];
 #pragma unroll
-      for (int e = 0; e < kLocUnroll; ++e) yv[e] = b[wd[e] & 0xFFFFu];
+      for (int e = 0; e < LU; ++e) yv[e] = e < lw ? b[wd[e] & 0xFFFFu] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int e = 0; e < kLocUnroll; ++e) {
+      for (int e = 0; e < LU; ++e) {
         const float av = __uint_as_float(wd[e] & 0xFFFF0000u);
         t0 += av * yv[e].x;
         t1 += av * yv[e].y;
         t2 += av * yv[e].z;
       }
-      for (int e = kLocUnroll; e < lw; ++e) {
+      for (int e = LU; e < lw; ++e) {
         const uint32_t word = le[e * NT];
         const float av = __uint_as_float(word & 0xFFFF0000u);
         const float4 y4 = b[word & 0xFFFFu];
@@ -440,7 +438,7 @@ __device__ __forceinline__ void coarse_solve(const float* s_Einv, const float* s
 }
 }  // namespace
 
-template <int RPT, bool COARSE>
+template <int RPT, bool COARSE, bool WIDE>
 __global__ void __launch_bounds__(NT, 1) pcg32_kernel(PcgArgsT<float> a, Pcg32Work wk) {
   constexpr int NC = COARSE ? kModes * NR : 0;
   constexpr int NV0 = 4 * NR + NC;  // gamma, delta, rr, bb, Phi^T w
@@ -479,10 +477,18 @@ __global__ void __launch_bounds__(NT, 1) pcg32_kernel(PcgArgsT<float> a, Pcg32Wo
     s_c1[threadIdx.x] = wk.c1[threadIdx.x];
     s_c2[threadIdx.x] = wk.c2[threadIdx.x];
   }
-  if (lw > 0) {
-    const uint32_t* __restrict__ lsrc = wk.loc + (size_t)blockIdx.x * RPT * lw * NT;
-    for (int e = threadIdx.x; e < RPT * lw * NT; e += NT) sLoc[e] = __ldg(lsrc + e);
-  }
+  constexpr bool kHold = RPT <= 2;
+  constexpr int kLU = WIDE ? kWideRows : kNarrowRows;
+  LocalPrec<RPT, kLU, kHold && !WIDE> lp;
+  lp.buf = sBuf;
+  lp.table = sLoc;
+  lp.c1 = s_c1;
+  lp.c2 = s_c2;
+  lp.c0 = wk.c0;
+  lp.lw = lw;
+  lp.degree = wk.degree;
+  lp.pb = 0;
+  lp.load(lw > 0 ? wk.loc + (size_t)blockIdx.x * RPT * lw * NT : nullptr);
 
   float x[RPT][NR], r[RPT][NR], p[RPT][NR], s[RPT][NR], u[RPT][NR], w[RPT][NR];
   float di[RPT], sd[RPT];
@@ -509,10 +515,9 @@ __global__ void __launch_bounds__(NT, 1) pcg32_kernel(PcgArgsT<float> a, Pcg32Wo
     }
   }
 
-  auto spmv = [&](const float4* __restrict__ z, float (&y)[RPT][NR]) {
-    spmv_rows_v<RPT, kGather>(rowptr, col, val, own, vr, z, y);
-  };
-  LocalPrec<RPT> lp{sBuf, sLoc, s_c1, s_c2, wk.c0, lw, wk.degree, 0};
+  MatRows<RPT, RPT <= 4 ? kLU : kGather, kHold> mat{rowptr, col, val};
+  mat.load(own, vr);
+  auto spmv = [&](const float4* __restrict__ z, float (&y)[RPT][NR]) { mat.mul(z, y); };
   // u = P r + Phi cc (P: the block-local polynomial, D^-1 without one), stored
   // for the neighbours; every thread of the block calls it
   auto precond = [&]() {
@@ -761,7 +766,7 @@ timeout:
 // no exchange: its products run on the block's rows in shared memory.
 // With the coarse space, M = P + Phi E^-1 Phi^T is a two-level additive
 // Schwarz preconditioner (degree 1: P = D^-1, plain Jacobi).
-template <int RPT>
+template <int RPT, bool WIDE>
 __global__ void __launch_bounds__(NT, 1) pcg32p_kernel(PcgArgsT<float> a, Pcg32Work wk) {
   constexpr int NC = kModes * NR;
   constexpr int NV0 = 4 * NR + NC;  // gamma, delta, rr, bb, Phi^T w
@@ -795,10 +800,18 @@ __global__ void __launch_bounds__(NT, 1) pcg32p_kernel(PcgArgsT<float> a, Pcg32W
     s_c1[threadIdx.x] = wk.c1[threadIdx.x];
     s_c2[threadIdx.x] = wk.c2[threadIdx.x];
   }
-  {
-    const uint32_t* __restrict__ lsrc = wk.loc + (size_t)blockIdx.x * RPT * lw * NT;
-    for (int e = threadIdx.x; e < RPT * lw * NT; e += NT) sLoc[e] = __ldg(lsrc + e);
-  }
+  constexpr bool kHold = RPT <= 2;
+  constexpr int kLU = WIDE ? kWideRows : kNarrowRows;
+  LocalPrec<RPT, kLU, kHold && !WIDE> lp;  // P, the block-local part of M (a Chebyshev polynomial of the block's diagonal block)
+  lp.buf = sBuf;
+  lp.table = sLoc;
+  lp.c1 = s_c1;
+  lp.c2 = s_c2;
+  lp.c0 = wk.c0;
+  lp.lw = lw;
+  lp.degree = wk.degree;
+  lp.pb = 0;
+  lp.load(lw > 0 ? wk.loc + (size_t)blockIdx.x * RPT * lw * NT : nullptr);
 
   float x[RPT][NR], r[RPT][NR], u[RPT][NR], w[RPT][NR], p[RPT][NR], s[RPT][NR], qv[RPT][NR], z[RPT][NR];
   float di[RPT], sd[RPT];  // D^-1 and D^-1/2 of the rows
@@ -826,9 +839,9 @@ __global__ void __launch_bounds__(NT, 1) pcg32p_kernel(PcgArgsT<float> a, Pcg32W
     }
   }
 
-  auto spmv = [&](const float4* __restrict__ zsrc, float (&y)[RPT][NR]) {
-    spmv_rows_v<RPT, kGatherPart>(rowptr, col, val, own, vr, zsrc, y);
-  };
+  MatRows<RPT, kLU, kHold> mat{rowptr, col, val};
+  mat.load(own, vr);
+  auto spmv = [&](const float4* __restrict__ zsrc, float (&y)[RPT][NR]) { mat.mul(zsrc, y); };
   auto phi_t = [&](const float (&y)[RPT][NR], float* loc) { phi_t_rows<RPT>(sPhi, own, y, loc); };
   auto coarse_cc = [&]() { coarse_solve4(s_Einv, s_rho, s_cc4); };  // s_cc4 = E^-1 s_rho
   // o[j] = sum_m rows[v][m] cc[m][j] for row k (rows: sPhi or sAPhi)
@@ -846,19 +859,37 @@ __global__ void __launch_bounds__(NT, 1) pcg32p_kernel(PcgArgsT<float> a, Pcg32W
     o[1] = acc.y;
     o[2] = acc.z;
   };
-  // out = P y, the block-local part of M (a Chebyshev polynomial of the block's diagonal block)
-  LocalPrec<RPT> lp{sBuf, sLoc, s_c1, s_c2, wk.c0, lw, wk.degree, 0};
   auto local_apply = [&](const float (&y)[RPT][NR], float (&out)[RPT][NR]) { lp.apply(own, di, sd, y, out); };
   auto rhs = [&](int k, int j) {  // b of row k (vertex order on input)
     return a.b[(int64_t)__ldg(perm + vr[k]) * NR + j];
   };
 
-  // ---- r = b - A x ------------------------------------------------------
+  // ---- r = b - A x, x gathered in place through the permutation (it is
+  // written back only after the barriers below)
 #pragma unroll
-  for (int k = 0; k < RPT; ++k)
-    if (own[k]) wk.ug[vr[k]] = make_float4(x[k][0], x[k][1], x[k][2], 0.f);
-  if (!gbar(wk, epoch, &s_flag, a.wait_ns)) goto timeout;
-  spmv(wk.ug, w);
+  for (int k = 0; k < RPT; ++k) {
+    w[k][0] = w[k][1] = w[k][2] = 0.f;
+    if (!own[k]) continue;
+    const int32_t e0 = __ldg(rowptr + vr[k]), e1 = __ldg(rowptr + vr[k] + 1);
+    for (int32_t e = e0; e < e1; e += 8) {
+      float av[8], x0[8], x1[8], x2[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const bool on = e + t < e1;
+        av[t] = on ? __ldg(val + e + t) : 0.f;
+        const float* xs = a.x + NR * (on ? (int64_t)__ldg(perm + __ldg(col + e + t)) : 0);
+        x0[t] = on ? __ldcg(xs) : 0.f;
+        x1[t] = on ? __ldcg(xs + 1) : 0.f;
+        x2[t] = on ? __ldcg(xs + 2) : 0.f;
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        w[k][0] += av[t] * x0[t];
+        w[k][1] += av[t] * x1[t];
+        w[k][2] += av[t] * x2[t];
+      }
+    }
+  }
 #pragma unroll
   for (int k = 0; k < RPT; ++k)
 #pragma unroll
@@ -1050,7 +1081,7 @@ constexpr size_t plain_smem(bool parted, int lw) {
          (parted ? 2 * sizeof(float4) * RPT * NT + sizeof(uint32_t) * (size_t)RPT * lw * NT : 0);
 }
 
-template <int RPT, bool C>
+template <int RPT, bool C, bool W>
 cudaError_t prepare32() {
   // above the default 48 KB the kernel needs the opt-in, a per-device attribute
   const size_t smem = plain_smem<RPT, C>(RPT <= 4, RPT <= 4 ? cg_local_width_max(RPT) : 0);
@@ -1063,13 +1094,13 @@ cudaError_t prepare32() {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (set[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(pcg32_kernel<RPT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(pcg32_kernel<RPT, C, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) set[dev] = true;
   return e;
 }
 
-template <int RPT, bool C>
-cudaError_t launch32(const PcgArgsT<float>& args, const Pcg32Work& work, int grid, cudaStream_t st) {
+template <int RPT, bool C, bool W>
+cudaError_t launch32w(const PcgArgsT<float>& args, const Pcg32Work& work, int grid, cudaStream_t st) {
   const bool parted = work.off != nullptr;
   const int lw = (parted && work.degree > 1) ? work.lw : 0;
   if (parted && (RPT > 4 || !work.perm || lw > cg_local_width_max(RPT) || (lw > 0 && !work.loc) ||
@@ -1079,7 +1110,14 @@ cudaError_t launch32(const PcgArgsT<float>& args, const Pcg32Work& work, int gri
   PcgArgsT<float> a = args;
   Pcg32Work w = work;
   void* params[] = {(void*)&a, (void*)&w};
-  return cudaLaunchCooperativeKernel((const void*)pcg32_kernel<RPT, C>, dim3(grid), dim3(NT), params, smem, st);
+  return cudaLaunchCooperativeKernel((const void*)pcg32_kernel<RPT, C, W>, dim3(grid), dim3(NT), params, smem, st);
+}
+
+template <int RPT, bool C>
+cudaError_t launch32(const PcgArgsT<float>& args, const Pcg32Work& work, int grid, cudaStream_t st) {
+  if constexpr (RPT <= 4)
+    if (work.off && work.lw > kNarrowRows) return launch32w<RPT, C, true>(args, work, grid, st);
+  return launch32w<RPT, C, false>(args, work, grid, st);
 }
 }  // namespace
 
@@ -1106,7 +1144,7 @@ constexpr size_t pipe_smem(int lw) {
          sizeof(uint32_t) * (size_t)RPT * lw * NT;
 }
 
-template <int RPT>
+template <int RPT, bool W>
 cudaError_t prepare32p() {
   static bool set[64] = {false};
   static std::mutex mu;  // handles may be built from several threads
@@ -1118,7 +1156,7 @@ cudaError_t prepare32p() {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (set[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(pcg32p_kernel<RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(pcg32p_kernel<RPT, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) set[dev] = true;
   return e;
 }
@@ -1130,8 +1168,8 @@ cudaError_t launch32p(const PcgArgsT<float>& args, const Pcg32Work& work, int gr
   const int lw = w.degree > 1 ? w.lw : 0;
   if (lw > cg_local_width_max(RPT) || (w.degree > 1 && !w.loc)) return cudaErrorInvalidValue;
   void* params[] = {(void*)&a, (void*)&w};
-  return cudaLaunchCooperativeKernel((const void*)pcg32p_kernel<RPT>, dim3(grid), dim3(NT), params, pipe_smem<RPT>(lw),
-                                     st);
+  const void* f = w.lw > kNarrowRows ? (const void*)pcg32p_kernel<RPT, true> : (const void*)pcg32p_kernel<RPT, false>;
+  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(NT), params, pipe_smem<RPT>(lw), st);
 }
 }  // namespace
 
@@ -1166,16 +1204,13 @@ cudaError_t launch_aphi32(int64_t n, const int32_t* rowptr, const int32_t* col, 
 }
 
 cudaError_t prepare_pcg32() {
-  cudaError_t e = prepare32<1, true>();
-  if (e == cudaSuccess) e = prepare32<1, false>();
-  if (e == cudaSuccess) e = prepare32<2, true>();
-  if (e == cudaSuccess) e = prepare32<2, false>();
-  if (e == cudaSuccess) e = prepare32<4, true>();
-  if (e == cudaSuccess) e = prepare32<4, false>();
-  if (e == cudaSuccess) e = prepare32<8, true>();
-  if (e == cudaSuccess) e = prepare32p<1>();
-  if (e == cudaSuccess) e = prepare32p<2>();
-  if (e == cudaSuccess) e = prepare32p<4>();
+  cudaError_t e = cudaSuccess;
+  auto all = [&](auto... f) { ((e = e == cudaSuccess ? f() : e), ...); };
+  all(prepare32<1, true, false>, prepare32<1, false, false>, prepare32<2, true, false>, prepare32<2, false, false>,
+      prepare32<4, true, false>, prepare32<4, false, false>, prepare32<8, true, false>, prepare32<1, true, true>,
+      prepare32<1, false, true>, prepare32<2, true, true>, prepare32<2, false, true>, prepare32<4, true, true>,
+      prepare32<4, false, true>, prepare32p<1, false>, prepare32p<2, false>, prepare32p<4, false>,
+      prepare32p<1, true>, prepare32p<2, true>, prepare32p<4, true>);
   return e;
 }
 

@@ -37,6 +37,7 @@
 
 #include "emu_internal.h"
 #include "emu_pcg.h"
+#include "emu_reduce.cuh"
 
 namespace emu {
 
@@ -100,26 +101,6 @@ __device__ __forceinline__ void vbar_exit(GridBarrier* bar) {
       atomicExch(&bar->v_err, 0u);
       atomicExch(&bar->v_done, 0u);
     }
-  }
-}
-
-// Halving butterfly of C values (a power of two) over one warp in a fixed
-// order: lane l ends with the sum of value (l * C / 32) in v[0].
-template <int C, int O>
-__device__ __forceinline__ void warp_halve(double* v, int lane) {
-  if constexpr (C >= 2) {
-    constexpr int H = C / 2;
-    const bool hi = (lane & O) != 0;
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-      const double send = hi ? v[i] : v[H + i];
-      const double keep = hi ? v[H + i] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-    }
-    if constexpr (O > 1) warp_halve<H, O / 2>(v, lane);
-  } else {
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-    if constexpr (O > 1) warp_halve<1, O / 2>(v, lane);
   }
 }
 
@@ -217,13 +198,13 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
   auto reduce = [&](const double (&d4)[4], double y) {
     if (data) {
       double t4[4] = {d4[0], d4[1], d4[2], d4[3]};
-      warp_halve<4, 16>(t4, lane);
+      warp_halve<4>(t4, lane);
       if ((lane & 7) == 0) s_red[warp * kRed + (lane >> 3)] = t4[0];
       if constexpr (COARSE) {
         double t[kModes];
 #pragma unroll
         for (int m = 0; m < kModes; ++m) t[m] = sPhi[m * rows + lr] * y;
-        warp_halve<kModes, 16>(t, lane);
+        warp_halve<kModes>(t, lane);
         if ((lane & 1) == 0) s_red[warp * kRed + 4 + (lane >> 1)] = t[0];
       }
     }
@@ -424,6 +405,241 @@ template <bool C> cudaError_t pick64(const PcgArgsT<double>& a, int rows, int gr
   return launch64<960, C>(a, rows, grid, threads, st);
 }
 }  // namespace
+
+// ------------------------------------------------- sixteen right-hand sides --
+// The same CG without a coarse space for 16 columns: the subspace iteration of
+// the low-rank basis (Eq. 9) and the joints' responses, at set-up. The generic
+// kernel gives a thread one row and 16 columns, about 550 FP64 instructions an
+// iteration at 64 cycles each (70 us at 1,485 rows, 45 of the 50 ms of a
+// 6,080-tet handle's set-up). Here a warp owns one column of 32 rows and a
+// block CPB columns of 128 rows, so the columns of a small system spread over
+// the SMs. Every value is formed by the generic kernel's operations in its
+// order (its blocks of ``per`` rows, its trees), so the basis, and with it
+// every later rounding of a solve, is the same to the last bit.
+constexpr int kNR16 = 16, kRows16 = 128;
+
+// blockIdx.x = (virtual block, column group); warp w: rows 32 (w % 4) .., column w / 4 of the group
+template <int CPB>
+__global__ void __launch_bounds__(kRows16* CPB, 2) pcg16_kernel(PcgArgsT<double> a, int per, int nvb) {
+  constexpr int kGroups = kNR16 / CPB;
+  __shared__ double sVal[kEll][kRows16];
+  __shared__ int32_t sCol[kEll][kRows16];
+  __shared__ double s_red[4 * CPB][4];
+  __shared__ double s_grp[4][4 * CPB];
+  __shared__ double s_al[CPB], s_be[CPB];
+  __shared__ int s_act[CPB], s_zero[CPB];
+  __shared__ int s_flag, s_any;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rw = warp & 3, jc = warp >> 2;
+  const int vb = blockIdx.x / kGroups, cg = blockIdx.x % kGroups, j = cg * CPB + jc;
+  const int64_t n = a.n;
+  const int64_t r0 = (int64_t)vb * per, r1 = r0 + per < n ? r0 + per : n;
+  const int nwr = r1 > r0 ? (int)((r1 - r0 + 31) / 32) : 0;
+  const int lr = rw * 32 + lane;
+  const bool own = r0 + lr < r1;
+  const int64_t v = own ? r0 + lr : 0;
+  double* __restrict__ ug = a.u + (size_t)j * n;
+  double* __restrict__ part = a.partials;  // [virtual block][item][column]
+  int* act = reinterpret_cast<int*>(part + (size_t)nvb * 64);  // per column group: still active
+  unsigned epoch = 0;
+  int cnt = 0;
+  int32_t e0 = 0, e1 = 0;
+  if (own) {
+    e0 = __ldg(a.rowptr + v);
+    e1 = __ldg(a.rowptr + v + 1);
+    cnt = e1 - e0;
+  }
+  for (int t = jc; t < kEll; t += CPB) {
+    sVal[t][lr] = t < cnt ? __ldg(a.val + e0 + t) : 0.0;
+    sCol[t][lr] = t < cnt ? __ldg(a.col + e0 + t) : 0;
+  }
+  const double di = own ? __ldg(a.dinv + v) : 0.0;
+  const double bv = own ? a.b[v * kNR16 + j] : 0.0;
+  double x = own ? a.x[v * kNR16 + j] : 0.0;
+  __syncthreads();
+  auto spmv = [&](const double* z, int64_t stride) -> double {  // entries in the row's order, one accumulator
+    double zz[kEll], acc = 0.0;
+#pragma unroll
+    for (int t = 0; t < kEll; ++t) zz[t] = t < cnt ? __ldcg(z + sCol[t][lr] * stride) : 0.0;
+#pragma unroll
+    for (int t = 0; t < kEll; ++t)
+      if (t < cnt) acc = fma(sVal[t][lr], zz[t], acc);
+    for (int32_t e = e0 + kEll; e < e1; ++e) acc = fma(__ldg(a.val + e), __ldcg(z + __ldg(a.col + e) * stride), acc);
+    return acc;
+  };
+  // block sums of four items of this column into the virtual block's partials
+  auto reduce = [&](double d0, double d1, double d2, double d3) {
+    double t4[4] = {d0, d1, d2, d3};
+    if (rw < nwr) {
+      warp_halve<4>(t4, lane);
+      if ((lane & 7) == 0) s_red[warp][lane >> 3] = t4[0];
+    }
+    __syncthreads();
+    if (tid < 4 * CPB) {
+      const int item = tid / CPB, c = tid % CPB;
+      double t = 0.0;
+      for (int g = 0; g < nwr; ++g) t += s_red[c * 4 + g][item];
+      __stcg(part + (size_t)vb * 64 + item * kNR16 + cg * CPB + c, t);
+    }
+  };
+  // sums over the virtual blocks: four groups take every fourth, then the
+  // groups in order; thread item * CPB + c returns item ``item`` of column c
+  auto gather_sums = [&]() -> double {
+    if (tid < 16 * CPB) {
+      const int k = tid % (4 * CPB), g = tid / (4 * CPB);
+      const double* src = part + (k / CPB) * kNR16 + cg * CPB + k % CPB;
+      double t = 0.0;
+      for (int b = g; b < nvb; b += 32) {
+        double l[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) l[q] = b + 4 * q < nvb ? __ldcg(src + (size_t)(b + 4 * q) * 64) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (b + 4 * q < nvb) t += l[q];
+      }
+      s_grp[g][k] = t;
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (tid < 4 * CPB)
+      for (int g = 0; g < 4; ++g) t += s_grp[g][tid];
+    __syncthreads();
+    return t;
+  };
+
+  double r = own ? bv - spmv(a.x + j, kNR16) : 0.0;
+  double u = di * r;
+  if (own) __stcg(ug + v, u);
+  if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+  {
+    double w = spmv(ug, 1);
+    reduce(r * u, w * u, r * r, bv * bv);
+    if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+    // the scalars of column c in thread c, from the sums of threads c, CPB + c, ..
+    double sga = 0.0, sal = 0.0, sthr = 0.0, sbb = 0.0, srr = 0.0;
+    int sact = 0;
+    double t = gather_sums();
+    {
+      const double dl = __shfl_sync(0xffffffffu, t, (lane + CPB) & 31), rr = __shfl_sync(0xffffffffu, t, (lane + 2 * CPB) & 31),
+                   bb = __shfl_sync(0xffffffffu, t, (lane + 3 * CPB) & 31);
+      if (tid < CPB) {
+        sbb = bb;
+        srr = rr;
+        sthr = a.tol * a.tol * bb;
+        sga = t;
+        sact = (rr <= sthr || !(dl > 0.0)) ? 0 : 1;
+        sal = sact ? t / dl : 0.0;
+        s_al[tid] = sal;
+        s_act[tid] = sact;
+        s_zero[tid] = bb == 0.0;
+      }
+    }
+    __syncthreads();
+    double p = u, s = w;
+    if (s_zero[jc]) x = 0.0;  // zero right-hand side: x = 0 exactly
+    int it = 0;
+    bool all_done = false;
+    for (;;) {
+      if (vb == 0 && tid == 0) {
+        int on = 0;
+        for (int c = 0; c < CPB; ++c) on |= s_act[c];
+        __stcg(act + cg, on);
+      }
+      if (s_act[jc] && it < a.max_iter) {
+        x = fma(s_al[jc], p, x);
+        r = fma(-s_al[jc], s, r);
+        u = di * r;
+      }
+      if (own) __stcg(ug + v, u);
+      if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+      // every block sees every group's state, so all leave together
+      if (tid == 0) {
+        int on = 0;
+        for (int g = 0; g < kGroups; ++g) on |= __ldcg(act + g);
+        s_any = on;
+      }
+      __syncthreads();
+      all_done = s_any == 0;
+      if (all_done || it >= a.max_iter) break;
+      ++it;
+      w = spmv(ug, 1);
+      reduce(r * u, w * u, r * r, 0.0);
+      if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
+      t = gather_sums();
+      {
+        const double dl = __shfl_sync(0xffffffffu, t, (lane + CPB) & 31), rr = __shfl_sync(0xffffffffu, t, (lane + 2 * CPB) & 31);
+        if (tid < CPB && sact) {
+          srr = rr;
+          if (rr <= sthr) {
+            sact = 0;
+          } else {
+            const double be = t / sga;
+            const double den = dl - be * t / sal;
+            if (!(den > 0.0)) {  // breakdown: stop this column
+              sact = 0;
+            } else {
+              s_be[tid] = be;
+              sal = t / den;
+              s_al[tid] = sal;
+              sga = t;
+            }
+          }
+          s_act[tid] = sact;
+        }
+      }
+      __syncthreads();
+      if (s_act[jc]) {
+        p = fma(s_be[jc], p, u);
+        s = fma(s_be[jc], s, w);
+      }
+      __syncthreads();
+    }
+    if (own) a.x[v * kNR16 + j] = x;
+    if (vb == 0 && tid < CPB && a.relres_out) a.relres_out[cg * CPB + tid] = sbb > 0.0 ? sqrt(srr / sbb) : 0.0;
+    if (blockIdx.x == 0 && tid == 0) {
+      if (a.iters_out) atomicAdd(a.iters_out, it);
+      if (a.fail_out && !all_done) atomicExch(a.fail_out, 1);
+      if (a.last_iters) *a.last_iters = it;
+    }
+  }
+  vbar_exit(a.bar);
+  return;
+timeout:
+  if (tid == 0 && a.timeout_out) atomicExch(a.timeout_out, 1);
+  vbar_exit(a.bar);
+}
+
+namespace {
+template <int CPB> cudaError_t launch16(const PcgArgsT<double>& args, int per, int nvb, cudaStream_t st) {
+  PcgArgsT<double> a = args;
+  void* params[] = {(void*)&a, (void*)&per, (void*)&nvb};
+  return cudaLaunchCooperativeKernel((const void*)pcg16_kernel<CPB>, dim3(nvb * (kNR16 / CPB)), dim3(kRows16 * CPB),
+                                     params, 0, st);
+}
+}  // namespace
+
+// Columns per block so that the grid is about two blocks per SM; 0 where the
+// 16 n threads of the kernel exceed 1,024 per SM, or the generic kernel's
+// blocks (``grid`` of them) would hold more than 128 rows.
+int pcg16_columns(int64_t n, int grid, int sms) {
+  if (grid < 1 || n < 1 || kNR16 * n > 1024 * (int64_t)sms || (n + grid - 1) / grid > kRows16) return 0;
+  for (int c = 1; c <= 4; c *= 2)
+    if ((int64_t)grid * (kNR16 / c) <= 2 * (int64_t)sms) return c;
+  return 0;
+}
+
+cudaError_t launch_pcg16(const PcgArgsT<double>& args, int grid, int columns, cudaStream_t st) {
+  if (!args.bar_clean) {
+    const cudaError_t e = cudaMemsetAsync(args.bar, 0, sizeof(GridBarrier), st);
+    if (e != cudaSuccess) return e;
+  }
+  const int per = (int)((args.n + grid - 1) / grid);
+  switch (columns) {
+    case 1: return launch16<1>(args, per, grid, st);
+    case 2: return launch16<2>(args, per, grid, st);
+    default: return launch16<4>(args, per, grid, st);
+  }
+}
 
 // Rows per block: the smallest multiple of 32 that needs at most one block
 // per SM; false above 320 (n > 320 per SM: the generic kernel).

@@ -4,23 +4,55 @@
 
 namespace emu {
 
+// Halving butterfly of C values (a power of two, at most 64) over one warp in
+// a fixed order: at each step a lane keeps half of its values and adds its
+// partner's copy of that half. Lane l ends with the sums of the values
+// warp_halve_first<C>(l) .. in v[0..max(C / 32, 1)). Every value's additions
+// pair the lanes as a plain xor tree does (the same bits), with about C adds a
+// lane instead of 5 C: on GB300 each FP64 warp instruction takes its warp 64
+// cycles, whatever its lanes or its neighbours do.
+template <int C, int O = 16>
+__device__ __forceinline__ void warp_halve(double* v, int lane) {
+  if constexpr (C >= 2) {
+    constexpr int H = C / 2;
+    const bool hi = (lane & O) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double send = hi ? v[i] : v[H + i];
+      const double keep = hi ? v[H + i] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    if constexpr (O > 1) warp_halve<H, O / 2>(v, lane);
+  } else {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+    if constexpr (O > 1) warp_halve<1, O / 2>(v, lane);
+  }
+}
+template <int C>
+__device__ __forceinline__ int warp_halve_first(int lane) {
+  if constexpr (C >= 32) return lane * (C / 32);
+  return lane / (32 / C);
+}
+__host__ __device__ constexpr int pow2_ceil(int x) { return x <= 1 ? 1 : 2 * pow2_ceil((x + 1) / 2); }
+
 // Sums v[0..NV) over the block (<= 256 threads) in a fixed order and writes
 // the NV totals to out[0..NV). Deterministic for a fixed launch shape.
 template <int NV>
 __device__ __forceinline__ void block_reduce_write(double (&v)[NV], double* out) {
-  __shared__ double sm[8 * NV];
+  constexpr int P = pow2_ceil(NV);
+  __shared__ double sm[8 * P];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double t[P];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double x = v[k];
+  for (int k = 0; k < P; ++k) t[k] = k < NV ? v[k] : 0.0;
+  warp_halve<P>(t, lane);
+  const int first = warp_halve_first<P>(lane);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) sm[warp * NV + k] = x;
-  }
+  for (int k = 0; k < (P >= 32 ? P / 32 : 1); ++k) sm[warp * P + first + k] = t[k];  // equal copies when P < 32
   __syncthreads();
   for (int k = threadIdx.x; k < NV; k += blockDim.x) {
     double x = 0.0;
-    for (int w = 0; w < nw; ++w) x += sm[w * NV + k];
+    for (int w = 0; w < nw; ++w) x += sm[w * P + k];
     out[k] = x;
   }
 }

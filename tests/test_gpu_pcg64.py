@@ -80,3 +80,27 @@ def test_coupling_solve_residual(name):
     np.testing.assert_array_equal(q[~free], Q[~free])
     scale = np.linalg.norm(np.where(free[:, None], b - K @ (Q * ~free[:, None]), Q))
     assert np.linalg.norm((b - K @ q)[free]) <= 1e-11 * scale
+
+
+# Set-up of the low-rank basis with one, two and four columns per block and on
+# the generic kernel (csrc/emu_pcg64.cu, pcg16_columns), with a full and a
+# ragged last block of 128 rows: a handle's first solve reaches its tolerance.
+SETUPS = {
+    "rows_128": lambda: box_beam(1, 1, 31),
+    "rows_132": lambda: box_beam(1, 1, 32),
+    "two_columns_3k": lambda: mtu_for_tet_count(12000),
+    "four_columns_9k": lambda: mtu_for_tet_count(40000),
+    "generic_13k": lambda: mtu_for_tet_count(60000),
+}
+
+
+@pytest.mark.parametrize("name", list(SETUPS))
+def test_first_solve_after_setup(name):
+    import paper_2006_08821_gb300 as emu
+
+    mesh = SETUPS[name]()
+    s = emu.Solver(mesh, emu.Params(precision=emu.PRECISION_MIXED))
+    s.set_activation(0.4)
+    st = s.solve()
+    assert st.status == 0 and st.rel_residual <= 1e-6
+    s.close()
