@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(256) k_bone_ls(BoneArgs a, const TQ* __restric
       for (int j = 0; j < kLsTrials; ++j) {
         const double x = sig * trM + sig * sig * e2 + sig * sig * sig * detM;
         if (x > -1.0) {
-          const double dl = log1p(x);
-          const double nh = sig * FFd + 0.5 * sig * sig * dd - sig * sig * e2 - sig * sig * sig * detM + x_minus_log1p(x);
+          const double xml = x_minus_log1p(x), dl = log1p_from(x, xml);
+          const double nh = sig * FFd + 0.5 * sig * sig * dd - sig * sig * e2 - sig * sig * sig * detM + xml;
           acc[j] += a.Vb[b] * (a.mu[b] * nh + 0.5 * a.lam[b] * dl * (2.0 * lnJ + dl));
         } else {
           acc[j] += 1e300;

@@ -46,9 +46,9 @@ __device__ void sym3_eig(const double* A, double* lam, double* W) {
       const int p = e == 2 ? 1 : 0, q = e == 0 ? 1 : 2, o = 3 - p - q;
       const double apq = a[p][q];
       if (apq == 0.0) continue;
-      const double theta = (a[q][q] - a[p][p]) / (2.0 * apq);
-      const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-      const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
+      const double theta = (a[q][q] - a[p][p]) * inv_n(2.0 * apq);
+      const double ta = inv_n(fabs(theta) + sqrt_n(theta * theta + 1.0)), t = copysign(ta, theta);
+      const double c = rsqrt_n(t * t + 1.0), s = t * c;
       const double aop = a[o][p], aoq = a[o][q];
       a[o][p] = a[p][o] = c * aop - s * aoq;
       a[o][q] = a[q][o] = s * aop + c * aoq;
@@ -134,13 +134,14 @@ __device__ void hessian_F(const double* F, double lnJ, const ElemMat<double>& md
   matmul3(R, Vm, U);
   ok = sig[0] > 0.0 && sig[1] > 0.0 && sig[2] > 0.0;
   const double cm = md.mu - md.lam * lnJ;
+  const double is[3] = {inv_n(sig[0]), inv_n(sig[1]), inv_n(sig[2])};
   // the 3 x 3 block on the diagonal entries
   double A3[9], eta[3], Wd[9];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      A3[3 * i + j] = md.lam / (sig[i] * sig[j]) + (i == j ? md.mu + cm / (sig[i] * sig[i]) : 0.0);
+      A3[3 * i + j] = md.lam * (is[i] * is[j]) + (i == j ? md.mu + cm * (is[i] * is[i]) : 0.0);
   sym3_eig(A3, eta, Wd);
   double z[9];
 #pragma unroll
@@ -159,7 +160,7 @@ __device__ void hessian_F(const double* F, double lnJ, const ElemMat<double>& md
 #pragma unroll
   for (int e = 0; e < 3; ++e) {
     const int i = e == 2 ? 1 : 0, j = e == 0 ? 1 : 2;
-    const double tw = cm / (sig[i] * sig[j]);
+    const double tw = cm * (is[i] * is[j]);
 #pragma unroll
     for (int sgn = 0; sgn < 2; ++sgn) {
       const double lam = sgn == 0 ? md.mu + tw : md.mu - tw;
@@ -192,8 +193,9 @@ __device__ __forceinline__ bool chol9(double* H) {
     double d = H[pk(j, j)];
 #pragma unroll
     for (int k = 0; k < j; ++k) d -= H[pk(j, k)] * H[pk(j, k)];
-    ok = ok && d > 0.0;
-    const double id = d > 0.0 ? 1.0 / sqrt(d) : 1.0;
+    const bool pos = positive_n(d);
+    ok = ok && pos;
+    const double id = pos ? rsqrt_n(d) : 1.0;
     H[pk(j, j)] = id;
 #pragma unroll
     for (int i = j + 1; i < 9; ++i) {
@@ -497,8 +499,8 @@ __global__ void __launch_bounds__(128) k_ls_fform(TetArgs<double> a, LsSelect se
       const double x = sig * trM + sig * sig * e2 + sig * sig * sig * detM;
       double dpsi;
       if (x > -1.0 && J > 0.0) {
-        const double dl = log1p(x);
-        const double nh = sig * FFd + 0.5 * sig * sig * dd - sig * sig * e2 - sig * sig * sig * detM + x_minus_log1p(x);
+        const double xml = x_minus_log1p(x), dl = log1p_from(x, xml);
+        const double nh = sig * FFd + 0.5 * sig * sig * dd - sig * sig * e2 - sig * sig * sig * detM + xml;
         dpsi = md.mu * nh + 0.5 * md.lam * dl * (2.0 * lnJ + dl) + md.ka * (2.0 * sig * Fudu + sig * sig * dudu);
         dpsi = dpsi * md.V - sig * dnu;
       } else {

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(128) k_grad(TetArgs<TW> a) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) yv[k] = (TW)g[k];
     apply_I_minus_N(U, yv);
-    const TW ic = (TW)(1.0 / c);
+    const TW ic = (TW)inv_n(c);
 #pragma unroll
     for (int k = 0; k < 9; ++k) a.y[k * m + i] = yv[k] * ic;
 #pragma unroll
@@ -245,24 +245,7 @@ template <typename TW> void launch_syrk(const TetArgs<TW>& a, int grid, double* 
 
 // ------------------------------------------- capacitance sum and solve ----
 __device__ __forceinline__ float pivot_inverse(float d) { return __frcp_rn(d); }
-// 1 / d in FP64 by Newton's iteration: the hardware estimate is good to 2^-20
-// or so, and one cubic step (error e -> e^3) leaves rounding. Three FP64 instructions; the range
-// test is on the exponent's integer bits (an FP64 comparison costs a warp as
-// much as a multiplication).
-__device__ __forceinline__ double pivot_inverse(double d) {
-  const int hi = __double2hiint(d);
-  if (!(hi > 0x01000000 && hi < 0x7e000000)) return 1.0 / d;  // outside 2^-1007 .. 2^993
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double e = fma(-d, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-__device__ __forceinline__ bool positive(float x) { return x > 0.f; }
-// x > 0 (false for NaN) on the bits
-__device__ __forceinline__ bool positive(double x) {
-  const long long b = __double_as_longlong(x);
-  return b > 0 && b <= 0x7ff0000000000000ll;
-}
+__device__ __forceinline__ double pivot_inverse(double d) { return inv_n(d); }
 
 constexpr int kCapLow = kK * (kK + 1) / 2;        // entries of the lower triangle
 constexpr int kCapSums = kCapLow + kK;            // and of B y
@@ -353,7 +336,7 @@ __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, i
   // warp), for the columns of the panel at p0; the four roots in four lanes
   auto substitute = [&](int p0, const T (*W)[kK + 1]) {
     const T d4 = W[lane & (kCapNB - 1)][p0 + (lane & (kCapNB - 1))];
-    const T ri4 = positive(d4) ? T(1) / sqrt(d4) : T(1);
+    const T ri4 = positive_n(d4) ? T(1) / sqrt(d4) : T(1);
     if (lane < kCapNB) sR[p0 + lane] = ri4;
 #pragma unroll
     for (int p = 0; p < kCapNB; ++p) {
@@ -385,7 +368,7 @@ __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, i
 #pragma unroll
       for (int p = 0; p < kCapNB; ++p) {
         T d = __shfl_sync(0xffffffffu, v[p], p);
-        if (!positive(d)) {  // not positive definite: recorded, z = 0 below
+        if (!positive_n(d)) {  // not positive definite: recorded, z = 0 below
           d = T(1);
           s_ok = 0;
         }
@@ -609,8 +592,8 @@ __global__ void __launch_bounds__(128) k_ls(TetArgs<TW> a, LsSelect sel) {
       double dpsi;
       if (x > -1.0) {
         // mu [s <F, d> + s^2 |d|^2 / 2 - log1p(x)] with log1p(x) = x - (x - log1p x)
-        const double dl = log1p(x);
-        const double nh = sig * FFd + 0.5 * sig * sig * dd - sig * sig * e2 - sig * sig * sig * detM + x_minus_log1p(x);
+        const double xml = x_minus_log1p(x), dl = log1p_from(x, xml);
+        const double nh = sig * FFd + 0.5 * sig * sig * dd - sig * sig * e2 - sig * sig * sig * detM + xml;
         dpsi = md.mu * nh + 0.5 * md.lam * dl * (2.0 * lnJ + dl) + md.ka * (2.0 * sig * Fudu + sig * sig * dudu);
         dpsi = dpsi * md.V - sig * dnu;
       } else {

@@ -121,30 +121,38 @@ constexpr int kLsNV = kLsTrials + 2;   // dPsi per trial + c<D,dD> + c|dD|^2
 // energy decrease is taken (not merely the first).
 __device__ __forceinline__ void ls_select_block(const double* dir_partials, int nblk_dir, const double* ls_partials, int nblk_ls,
                                 DevScalars* sc, double sigma0, double rho, double c_armijo) {
-  __shared__ double s_gtd[1], s_v[kLsNV];
-  block_sum_partials<1>(dir_partials, nblk_dir, s_gtd);
-  block_sum_partials<kLsNV>(ls_partials, nblk_ls, s_v);
-  if (threadIdx.x != 0) return;
-  const double gtd = s_gtd[0];
-  double v[kLsNV];
-  for (int k = 0; k < kLsNV; ++k) v[k] = s_v[k];
-  sc->gtd = gtd;
-  double sig = sc->sigma_start;
-  int accepted = -1;
-  double dE = 0.0;
-  if (gtd < 0.0) {
-    double s_j = sig, best_sig = sig;
-    for (int j = 0; j < kLsTrials; ++j) {
-      const double dEj = v[j] + s_j * v[kLsTrials] + 0.5 * s_j * s_j * v[kLsTrials + 1];
-      if (dEj <= c_armijo * s_j * gtd && (accepted < 0 || dEj < dE)) {
-        accepted = j;
-        dE = dEj;
-        best_sig = s_j;
-      }
-      s_j *= rho;
-    }
-    sig = best_sig;
+  // the direction's g . d and the line search's sums in one reduction
+  __shared__ double s_v[kLsNV + 1];
+  {
+    double v[kLsNV + 1];
+    thread_sum_partials<kLsNV>(ls_partials, nblk_ls, v);
+    thread_sum_partials<1>(dir_partials, nblk_dir, v + kLsNV);
+    block_reduce_write<kLsNV + 1>(v, s_v);
   }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  // trial j in lane j; lane 0 then picks in trial order
+  const double gtd = s_v[kLsNV], sig0 = sc->sigma_start;
+  const int j = threadIdx.x & (kLsTrials - 1);
+  double s_j = sig0;
+  for (int k = 0; k < kLsTrials - 1; ++k)
+    if (k < j) s_j *= rho;
+  const double dEj = s_v[j] + s_j * s_v[kLsTrials] + 0.5 * s_j * s_j * s_v[kLsTrials + 1];
+  const unsigned meets = __ballot_sync(0xffffffffu, dEj <= c_armijo * s_j * gtd);
+  double sig = sig0, dE = 0.0;
+  int accepted = -1;
+#pragma unroll
+  for (int k = 0; k < kLsTrials; ++k) {
+    const double dk = __shfl_sync(0xffffffffu, dEj, k), sk = __shfl_sync(0xffffffffu, s_j, k);
+    if (((meets >> k) & 1u) && (accepted < 0 || dk < dE)) {
+      accepted = k;
+      dE = dk;
+      sig = sk;
+    }
+  }
+  if (!(gtd < 0.0)) accepted = -1;
+  if (threadIdx.x != 0) return;
+  sc->gtd = gtd;
   if (accepted >= 0) {
     sc->sigma = sig;
     sc->sigma_start = sigma0;

@@ -21,6 +21,58 @@ namespace emu {
 
 template <typename T> EMU_HD T rsqrt2() { return T(0.70710678118654752440); }
 
+// 1 / x, 1 / sqrt(x), sqrt(x) in FP64. On the device Newton's iteration from the hardware's estimates (good to about
+// 2^-20; one cubic step leaves an ulp or so): a warp instruction of FP64 costs
+// its warp 64 cycles on GB300, and a division or square root is some twenty of
+// them where these take three to eight. Arguments near the ends of the range
+// (tested on the exponent bits) take the plain expressions.
+EMU_HD bool positive_n(float x) { return x > 0.f; }
+EMU_HD bool positive_n(double x) {  // x > 0 (false for NaN), on the bits on the device
+#ifdef __CUDA_ARCH__
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+#else
+  return x > 0.0;
+#endif
+}
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ bool mid_range(double x) {  // 2^-500 < x < 2^500
+  const int hi = __double2hiint(x);
+  return hi > 0x20b00000 && hi < 0x5f300000;
+}
+#endif
+EMU_HD double inv_n(double x) {
+#ifdef __CUDA_ARCH__
+  if (mid_range(fabs(x))) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+  }
+#endif
+  return 1.0 / x;
+}
+EMU_HD double rsqrt_n(double x) {
+#ifdef __CUDA_ARCH__
+  if (mid_range(x)) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x * r, r, 1.0);
+    return fma(r * e, fma(0.375, e, 0.5), r);
+  }
+#endif
+  return 1.0 / sqrt(x);
+}
+EMU_HD double sqrt_n(double x) {
+#ifdef __CUDA_ARCH__
+  if (mid_range(x)) {
+    const double r = rsqrt_n(x), s = x * r;
+    return fma(0.5 * r, fma(-s, s, x), s);
+  }
+#endif
+  return sqrt(x);
+}
+
 // ---------------------------------------------------------------- 3x3 ------
 template <typename T> EMU_HD T det3(const T* A) {
   return A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) +
@@ -34,6 +86,24 @@ template <typename T> EMU_HD T inv3(const T* A, T* B) {
   T c02 = A[3] * A[7] - A[4] * A[6];
   T det = A[0] * c00 + A[1] * c01 + A[2] * c02;
   T id = T(1) / det;
+  B[0] = c00 * id;
+  B[1] = (A[2] * A[7] - A[1] * A[8]) * id;
+  B[2] = (A[1] * A[5] - A[2] * A[4]) * id;
+  B[3] = c01 * id;
+  B[4] = (A[0] * A[8] - A[2] * A[6]) * id;
+  B[5] = (A[2] * A[3] - A[0] * A[5]) * id;
+  B[6] = c02 * id;
+  B[7] = (A[1] * A[6] - A[0] * A[7]) * id;
+  B[8] = (A[0] * A[4] - A[1] * A[3]) * id;
+  return det;
+}
+
+EMU_HD double inv3(const double* A, double* B) {
+  double c00 = A[4] * A[8] - A[5] * A[7];
+  double c01 = A[5] * A[6] - A[3] * A[8];
+  double c02 = A[3] * A[7] - A[4] * A[6];
+  double det = A[0] * c00 + A[1] * c01 + A[2] * c02;
+  double id = inv_n(det);
   B[0] = c00 * id;
   B[1] = (A[2] * A[7] - A[1] * A[8]) * id;
   B[2] = (A[1] * A[5] - A[2] * A[4]) * id;
@@ -380,6 +450,137 @@ template <typename T> EMU_HD void chart_factor(const T* R, const T* S, const T* 
         Uw[9 * i + 3 * r + b] = Wf[9 * i + b] * R[3 * r] + Wf[9 * i + 3 + b] * R[3 * r + 1] + Wf[9 * i + 6 + b] * R[3 * r + 2];
 }
 
+// chol in FP64 with the Newton roots above; idiag receives 1 / L_jj.
+template <int N> EMU_HD bool chol_n(double* A, double* idiag) {
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    double d = A[N * j + j];
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if (k < j) d -= A[N * j + k] * A[N * j + k];
+    const bool pos = positive_n(d);
+    ok = ok & pos;
+    const double id = pos ? rsqrt_n(d) : 1.0;
+    A[N * j + j] = pos ? d * id : 1.0;
+    idiag[j] = id;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if (i > j) {
+        double v = A[N * i + j];
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+          if (k < j) v -= A[N * i + k] * A[N * j + k];
+        A[N * i + j] = v * id;
+      }
+    }
+  }
+  return ok;
+}
+
+// The chart factor in FP64 (same factor, fewer operations).
+EMU_HD void chart_factor(const double* R, const double* S, const double* M6, double c, double* Uw, bool& ok) {
+  using T = double;
+  // Zr: 6 x 9, column (a,b) = stretch coords of e_a e_b^T (rotated frame)
+  T Kinv[9];
+  {
+    T tr = S[0] + S[4] + S[8];
+    T Km[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) Km[i] = -S[i];
+    Km[0] += tr;
+    Km[4] += tr;
+    Km[8] += tr;
+    inv3(Km, Kinv);
+  }
+  // Y = e_a e_b^T has k = 0 when a = b and k = +-e_c otherwise, so w is
+  // +-column c of Kinv; the three [w]x S are formed once (their stretch
+  // coordinates ws[c]) and each column of Zr is s(sym Y) -+ ws[c].
+  T ws[3][6];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const T w0 = Kinv[c], w1 = Kinv[3 + c], w2 = Kinv[6 + c];
+    // [w]x S ; [w]x = [[0,-w2,w1],[w2,0,-w0],[-w1,w0,0]]
+    T Wm[9];
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+      Wm[cc] = -w2 * S[3 + cc] + w1 * S[6 + cc];
+      Wm[3 + cc] = w2 * S[cc] - w0 * S[6 + cc];
+      Wm[6 + cc] = -w1 * S[cc] + w0 * S[3 + cc];
+    }
+    s_from_mat(Wm, ws[c]);
+  }
+  const T h = rsqrt2<T>();
+  // L_M = chol(M)
+  T LM[36], id[6];
+#pragma unroll
+  for (int i = 0; i < 36; ++i) LM[i] = M6[i];
+  ok = chol_n<6>(LM, id);
+  T Wf[54];
+  // Every column of Zr is a unit vector e_k (k < 3) or a pair
+  // h e_k +- ws[c], so with A = L_M^T, B = L_M^T ws the products are
+  // W W^T = A A^T + 2 B B^T (2 h^2 = 1) and U's columns are sums of L2^-1 A
+  // and L2^-1 B: a third fewer FP64 instructions than the 9-column form
+  // above.
+  T B[18];
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+      T acc = T(0);
+#pragma unroll
+      for (int k = i; k < 6; ++k) acc += LM[6 * k + i] * ws[cc][k];
+      B[3 * i + cc] = acc;
+    }
+  T K2[36];
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j) {
+      T acc = B[3 * i] * B[3 * j] + B[3 * i + 1] * B[3 * j + 1] + B[3 * i + 2] * B[3 * j + 2];
+      acc += acc;
+#pragma unroll
+      for (int k = i; k < 6; ++k) acc += LM[6 * k + i] * LM[6 * k + j];
+      if (i == j) acc += c;
+      K2[6 * i + j] = acc;
+      K2[6 * j + i] = acc;
+    }
+  ok = chol_n<6>(K2, id) && ok;
+  T SA[6][6], SB[3][6];  // columns of L2^-1 A and L2^-1 B
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) SA[k][i] = i <= k ? LM[6 * k + i] : T(0);
+    fwd_sub_inv<T, 6>(K2, id, SA[k]);
+  }
+#pragma unroll
+  for (int cc = 0; cc < 3; ++cc) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) SB[cc][i] = B[3 * i + cc];
+    fwd_sub_inv<T, 6>(K2, id, SB[cc]);
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    Wf[9 * i] = SA[0][i];
+    Wf[9 * i + 4] = SA[1][i];
+    Wf[9 * i + 8] = SA[2][i];
+    Wf[9 * i + 1] = h * SA[5][i] + SB[2][i];
+    Wf[9 * i + 3] = h * SA[5][i] - SB[2][i];
+    Wf[9 * i + 2] = h * SA[4][i] - SB[1][i];
+    Wf[9 * i + 6] = h * SA[4][i] + SB[1][i];
+    Wf[9 * i + 5] = h * SA[3][i] + SB[0][i];
+    Wf[9 * i + 7] = h * SA[3][i] - SB[0][i];
+  }
+  // world frame: Uw[:, (r,b)] = sum_a U[:, (a,b)] R[r][a]
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        Uw[9 * i + 3 * r + b] = Wf[9 * i + b] * R[3 * r] + Wf[9 * i + 3 + b] * R[3 * r + 1] + Wf[9 * i + 6 + b] * R[3 * r + 2];
+}
+
 // x <- x - Uw^T (Uw x)   (applies I - N to a world-frame 9-vector)
 template <typename T> EMU_HD void apply_I_minus_N(const T* Uw, T* x) {
   T t[6];
@@ -426,6 +627,46 @@ template <typename T> EMU_HD int polar_rotation(const T* X0, T* R, T tol, int ma
       for (int c = 0; c < 3; ++c) {
         T nx = T(0.5) * (g * X[3 * r + c] + ig * Xi[3 * c + r]);
         T dd = nx - X[3 * r + c];
+        diff += dd * dd;
+        X[3 * r + c] = nx;
+      }
+    if (diff <= tol * tol && it >= 1) {
+      ++it;
+      break;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) R[i] = X[i];
+  return it;
+}
+
+// The same in FP64 without the scaling (a cube root and two divisions) near
+// det = 1, where the plain iteration converges in the same count.
+EMU_HD int polar_rotation(const double* X0, double* R, double tol, int max_iter) {
+  double X[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) X[i] = X0[i];
+  int it = 0;
+  for (; it < max_iter; ++it) {
+    double Xi[9];
+    double det = inv3(X, Xi);
+    // determinant scaling while it matters: near det = 1 the plain iteration
+    // converges in the same count
+    double g = 1.0, ig = 1.0;
+    if (it < 4) {
+      double ad = det > 0.0 ? det : -det;
+      if (!(ad > 0.7 && ad < 1.4)) {
+        g = 1.0 / cbrt(ad);
+        ig = 1.0 / g;
+      }
+    }
+    double diff = 0.0;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        double nx = 0.5 * (g * X[3 * r + c] + ig * Xi[3 * c + r]);
+        double dd = nx - X[3 * r + c];
         diff += dd * dd;
         X[3 * r + c] = nx;
       }
@@ -546,6 +787,10 @@ EMU_HD float x_minus_log1p(float x) {
   }
   return x - log1pf(x);
 }
+
+// log1p(x) from x - log1p(x) where that came from the series (|x| < 0.05: the
+// difference is below x^2, so the subtraction keeps every bit of the result).
+EMU_HD double log1p_from(double x, double xml) { return fabs(x) < 0.05 ? x - xml : log1p(x); }
 
 // FP64: the series up to x^20 for |x| < 0.05 (next term below 0.05^19 relative).
 EMU_HD double x_minus_log1p(double x) {
