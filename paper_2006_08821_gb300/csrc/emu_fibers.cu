@@ -46,16 +46,20 @@ __global__ void __launch_bounds__(256) k_fiber_grad(int64_t m, const int4* __res
   }
 }
 
+// One device allocation for all arrays of a call (each cudaMalloc and cudaFree
+// costs tens of microseconds): sizes first, then the addresses.
 struct DevMem {
-  std::vector<void*> ptrs;
-  template <typename T> T* get(size_t count) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, std::max<size_t>(count * sizeof(T), 256)) != cudaSuccess) return nullptr;
-    ptrs.push_back(p);
-    return static_cast<T*>(p);
+  size_t bytes = 0;
+  char* base = nullptr;
+  size_t add(size_t b) {
+    const size_t at = bytes;
+    bytes += (std::max<size_t>(b, 1) + 255) & ~size_t(255);
+    return at;
   }
+  bool alloc() { return cudaMalloc(reinterpret_cast<void**>(&base), bytes) == cudaSuccess; }
+  template <typename T> T* at(size_t off) const { return reinterpret_cast<T*>(base + off); }
   ~DevMem() {
-    for (void* p : ptrs) cudaFree(p);
+    if (base) cudaFree(base);
   }
 };
 
@@ -82,7 +86,7 @@ extern "C" int emu_fiber_field(int64_t n_verts, const double* rest_pos, int64_t 
     if (dir[insertion[k]] == -1) return fiber_fail(EMU_ERR_INVALID_ARG, "a vertex is both origin and insertion");
     dir[insertion[k]] = 1;
   }
-  // rest geometry (D_m^-1 component-major, V) and the Laplacian's triplets
+  // rest geometry (D_m^-1 component-major, V)
   std::vector<double> Dinv(9 * m), V(m);
   std::vector<uint8_t> in_tet(n, 0);
   for (int64_t i = 0; i < m; ++i) {
@@ -106,65 +110,79 @@ extern "C" int emu_fiber_field(int64_t n_verts, const double* rest_pos, int64_t 
     V[i] = std::fabs(det) / 6.0;
     for (int k = 0; k < 4; ++k) in_tet[t[k]] = 1;
   }
-  std::vector<std::pair<int64_t, double>> trip;
-  trip.reserve(16 * m + n);
-  std::vector<double> rhs(3 * n, 0.0);
-  for (int64_t i = 0; i < m; ++i) {
-    const int32_t* t = tets + 4 * i;
-    double gN[4][3];
-    for (int k = 0; k < 3; ++k)
-      for (int c = 0; c < 3; ++c) gN[k][c] = Dinv[(3 * k + c) * m + i];
-    for (int c = 0; c < 3; ++c) gN[3][c] = -(gN[0][c] + gN[1][c] + gN[2][c]);
-    for (int a = 0; a < 4; ++a) {
-      if (dir[t[a]] != 0) continue;
-      for (int b = 0; b < 4; ++b) {
-        const double lv = V[i] * (gN[a][0] * gN[b][0] + gN[a][1] * gN[b][1] + gN[a][2] * gN[b][2]);
-        if (dir[t[b]] != 0)
-          rhs[3 * t[a]] -= lv * (double)dir[t[b]];
-        else
-          trip.push_back({(int64_t)t[a] * n + t[b], lv});
-      }
-    }
+  // The Laplacian row by row: a vertex's tets in order, each neighbour's place
+  // in the row remembered by vertex (a sort of all 16 m entries by key took
+  // most of the call before).
+  std::vector<int32_t> sptr(n + 1, 0), slot(4 * m);
+  for (int64_t k = 0; k < 4 * m; ++k) ++sptr[tets[k] + 1];
+  for (int64_t v = 0; v < n; ++v) sptr[v + 1] += sptr[v];
+  {
+    std::vector<int32_t> at(sptr.begin(), sptr.end() - 1);
+    for (int64_t k = 0; k < 4 * m; ++k) slot[at[tets[k]]++] = (int32_t)k;
   }
-  for (int64_t v = 0; v < n; ++v)
+  std::vector<double> rhs(3 * n, 0.0), dinv(n, 1.0), val;
+  std::vector<int32_t> rowptr(n + 1, 0), col, place(n, -1);
+  col.reserve(16 * n);
+  val.reserve(16 * n);
+  std::vector<std::pair<int32_t, double>> rowbuf;
+  for (int64_t v = 0; v < n; ++v) {
+    rowbuf.clear();
     if (dir[v] != 0 || !in_tet[v]) {
-      trip.push_back({v * n + v, 1.0});
+      rowbuf.push_back({(int32_t)v, 1.0});
       rhs[3 * v] = (double)dir[v];
+    } else {
+      for (int32_t k = sptr[v]; k < sptr[v + 1]; ++k) {
+        const int64_t i = slot[k] / 4;
+        const int a = slot[k] % 4;
+        double gN[4][3];
+        for (int r = 0; r < 3; ++r)
+          for (int c = 0; c < 3; ++c) gN[r][c] = Dinv[(3 * r + c) * m + i];
+        for (int c = 0; c < 3; ++c) gN[3][c] = -(gN[0][c] + gN[1][c] + gN[2][c]);
+        for (int b = 0; b < 4; ++b) {
+          const int32_t w = tets[4 * i + b];
+          const double lv = V[i] * (gN[a][0] * gN[b][0] + gN[a][1] * gN[b][1] + gN[a][2] * gN[b][2]);
+          if (dir[w] != 0) {
+            rhs[3 * v] -= lv * (double)dir[w];
+            continue;
+          }
+          if (place[w] < 0) {
+            place[w] = (int32_t)rowbuf.size();
+            rowbuf.push_back({w, 0.0});
+          }
+          rowbuf[place[w]].second += lv;
+        }
+      }
+      for (const auto& e : rowbuf) place[e.first] = -1;
+      std::sort(rowbuf.begin(), rowbuf.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
     }
-  std::sort(trip.begin(), trip.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
-  std::vector<int32_t> rowptr(n + 1, 0), col;
-  std::vector<double> val, dinv(n, 1.0);
-  col.reserve(trip.size());
-  val.reserve(trip.size());
-  for (size_t k = 0; k < trip.size();) {
-    const int64_t key = trip[k].first;
-    double s = 0.0;
-    while (k < trip.size() && trip[k].first == key) s += trip[k++].second;
-    const int64_t r = key / n, c = key % n;
-    col.push_back((int32_t)c);
-    val.push_back(s);
-    rowptr[r + 1]++;
-    if (r == c) dinv[r] = s > 0.0 ? 1.0 / s : 1.0;
+    for (const auto& e : rowbuf) {
+      col.push_back(e.first);
+      val.push_back(e.second);
+      if (e.first == v) dinv[v] = e.second > 0.0 ? 1.0 / e.second : 1.0;
+    }
+    rowptr[v + 1] = (int32_t)col.size();
   }
-  for (int64_t v = 0; v < n; ++v) rowptr[v + 1] += rowptr[v];
   const int64_t nnz = (int64_t)col.size();
 
   // device solve (3 columns of the CG kernel; columns 1 and 2 are zero)
   cudaStream_t st = (cudaStream_t)stream;
   const int grid = pcg_max_grid(3, n);
   DevMem dm;
-  int32_t *d_rowptr = dm.get<int32_t>(n + 1), *d_col = dm.get<int32_t>(nnz);
-  double *d_val = dm.get<double>(nnz), *d_dinv = dm.get<double>(n), *d_b = dm.get<double>(3 * n),
-         *d_x = dm.get<double>(3 * n), *d_r = dm.get<double>(3 * n), *d_u = dm.get<double>(3 * n),
-         *d_w = dm.get<double>(3 * n), *d_p = dm.get<double>(3 * n), *d_s = dm.get<double>(3 * n),
-         *d_part = dm.get<double>((size_t)std::max(grid, device_sms()) * 64), *d_D = dm.get<double>(9 * m),
-         *d_out = dm.get<double>(3 * m);
-  int4* d_tet = dm.get<int4>(m);
-  GridBarrier* d_bar = dm.get<GridBarrier>(1);
-  int* d_cnt = dm.get<int>(4);
-  if (!d_rowptr || !d_col || !d_val || !d_dinv || !d_b || !d_x || !d_r || !d_u || !d_w || !d_p || !d_s || !d_part ||
-      !d_D || !d_out || !d_tet || !d_bar || !d_cnt)
-    return fiber_fail(EMU_ERR_OOM, "device allocation failed");
+  const size_t o_rowptr = dm.add(4 * (n + 1)), o_col = dm.add(4 * nnz), o_val = dm.add(8 * nnz), o_dinv = dm.add(8 * n),
+               o_b = dm.add(24 * n), o_x = dm.add(24 * n), o_r = dm.add(24 * n), o_u = dm.add(24 * n),
+               o_w = dm.add(24 * n), o_p = dm.add(24 * n), o_s = dm.add(24 * n),
+               o_part = dm.add(8 * 64 * (size_t)std::max(grid, device_sms())), o_D = dm.add(72 * m),
+               o_out = dm.add(24 * m), o_tet = dm.add(16 * m), o_bar = dm.add(sizeof(GridBarrier)),
+               o_cnt = dm.add(4 * sizeof(int));
+  if (!dm.alloc()) return fiber_fail(EMU_ERR_OOM, "device allocation failed");
+  int32_t *d_rowptr = dm.at<int32_t>(o_rowptr), *d_col = dm.at<int32_t>(o_col);
+  double *d_val = dm.at<double>(o_val), *d_dinv = dm.at<double>(o_dinv), *d_b = dm.at<double>(o_b),
+         *d_x = dm.at<double>(o_x), *d_r = dm.at<double>(o_r), *d_u = dm.at<double>(o_u), *d_w = dm.at<double>(o_w),
+         *d_p = dm.at<double>(o_p), *d_s = dm.at<double>(o_s), *d_part = dm.at<double>(o_part),
+         *d_D = dm.at<double>(o_D), *d_out = dm.at<double>(o_out);
+  int4* d_tet = dm.at<int4>(o_tet);
+  GridBarrier* d_bar = dm.at<GridBarrier>(o_bar);
+  int* d_cnt = dm.at<int>(o_cnt);
   cudaError_t e = cudaSuccess;
   auto up = [&](void* dst, const void* src, size_t bytes) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);

@@ -36,6 +36,7 @@
 #include <mutex>
 
 #include "emu_internal.h"
+#include "emu_math.cuh"
 #include "emu_pcg.h"
 #include "emu_reduce.cuh"
 
@@ -119,8 +120,10 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
   __shared__ int s_flag;
   extern __shared__ double dyn[];
   double* sVal = dyn;                        // [kEll][rows]
-  double* sPhi = sVal + kEll * rows;         // [16][rows] when COARSE
-  int32_t* sCol = reinterpret_cast<int32_t*>(sPhi + NC * rows);  // [kEll][rows]
+  double* sPhi = sVal + kEll * rows;         // [16][rows + 1] when COARSE
+  const int ps = rows + 1;                   // its stride: sixteen modes of a row in sixteen banks
+  double* sW = sPhi + NC * ps;               // [warp][32] when COARSE
+  int32_t* sCol = reinterpret_cast<int32_t*>(sW + (COARSE ? NR * rows : 0));  // [kEll][rows]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = gridDim.x;
   const int64_t n = a.n;
@@ -149,7 +152,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
       sCol[t * rows + lr] = own && t < cnt ? __ldg(a.col + e0 + t) : (int32_t)v;
     }
     if constexpr (COARSE)
-      for (int m = j; m < kModes; m += NR) sPhi[m * rows + lr] = own ? __ldg(a.phit + (size_t)m * n + v) : 0.0;
+      for (int m = j; m < kModes; m += NR) sPhi[m * ps + lr] = own ? __ldg(a.phit + (size_t)m * n + v) : 0.0;
   }
   const double di = own ? __ldg(a.dinv + v) : 0.0;
   const double bv = own ? a.b[v * NR + j] : 0.0;
@@ -160,7 +163,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
   auto spmv = [&](const double* z, int64_t stride, int64_t plane) -> double {
     if (!own) return 0.0;
     const double* zj = z + j * plane;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    double acc = 0.0;  // one chain: an FP64 instruction occupies its warp as long as it takes
     constexpr int GW = MAXT > 512 ? 8 : 16;  // gathers in flight
 #pragma unroll
     for (int t0 = 0; t0 < kEll; t0 += GW) {
@@ -168,7 +171,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
 #pragma unroll
       for (int t = 0; t < GW; ++t) zz[t] = t0 + t < cnt ? __ldcg(zj + sCol[(t0 + t) * rows + lr] * stride) : 0.0;
 #pragma unroll
-      for (int t = 0; t < GW; ++t) acc[t & 3] = fma(sVal[(t0 + t) * rows + lr], zz[t], acc[t & 3]);
+      for (int t = 0; t < GW; ++t) acc = fma(sVal[(t0 + t) * rows + lr], zz[t], acc);
     }
     for (int32_t e = e0 + kEll; e < e1; e += 4) {  // long rows
       double av[4], zz[4];
@@ -179,20 +182,20 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
         zz[t] = on ? __ldcg(zj + __ldg(a.col + e + t) * stride) : 0.0;
       }
 #pragma unroll
-      for (int t = 0; t < 4; ++t) acc[t] = fma(av[t], zz[t], acc[t]);
+      for (int t = 0; t < 4; ++t) acc = fma(av[t], zz[t], acc);
     }
-    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    return acc;
   };
   // u = D^-1 r + Phi' rho
   auto precond = [&](double r) -> double {
-    double acc[4] = {di * r, 0.0, 0.0, 0.0};
+    double acc = di * r;
     if constexpr (COARSE) {
       if (data) {
 #pragma unroll
-        for (int m = 0; m < kModes; ++m) acc[m & 3] = fma(sPhi[m * rows + lr], s_rho[j * kModes + m], acc[m & 3]);
+        for (int m = 0; m < kModes; ++m) acc = fma(sPhi[m * ps + lr], s_rho[j * kModes + m], acc);
       }
     }
-    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    return acc;
   };
   // block sums of d4 (gamma, delta, rr, bb of this thread) and Phi'^T y, written as this block's partials
   auto reduce = [&](const double (&d4)[4], double y) {
@@ -201,11 +204,19 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
       warp_halve<4>(t4, lane);
       if ((lane & 7) == 0) s_red[warp * kRed + (lane >> 3)] = t4[0];
       if constexpr (COARSE) {
-        double t[kModes];
+        // mode lane % 16 over half of the warp's rows in each half of the warp:
+        // 17 FP64 instructions (16 products and a halving butterfly are 32)
+        double* sw = sW + warp * 32;
+        sw[lane] = y;
+        __syncwarp();
+        const double* ph = sPhi + (lane & 15) * ps + grp * 32 + (lane & 16);
+        const double* yw = sw + (lane & 16);
+        double t = 0.0;
 #pragma unroll
-        for (int m = 0; m < kModes; ++m) t[m] = sPhi[m * rows + lr] * y;
-        warp_halve<kModes>(t, lane);
-        if ((lane & 1) == 0) s_red[warp * kRed + 4 + (lane >> 1)] = t[0];
+        for (int q = 0; q < 16; ++q) t = fma(ph[q], yw[q], t);
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        if (lane < 16) s_red[warp * kRed + 4 + lane] = t;
+        __syncwarp();
       }
     }
     __syncthreads();
@@ -224,18 +235,13 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
     const int k = tid & (kPart - 1), g = tid / kPart, NG = (int)blockDim.x / kPart;
     if (k < 12 + NR * NC && g < NG) {
       double t = 0.0;
-      int b = g;
-      for (; b + 7 * NG < G; b += 8 * NG) {
+      for (int b = g; b < G; b += 8 * NG) {
         double l[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) l[q] = __ldcg(part + (size_t)(b + q * NG) * kPart + k);
-        t += ((l[0] + l[1]) + (l[2] + l[3])) + ((l[4] + l[5]) + (l[6] + l[7]));
-      }
-      if (b < G) {  // the rest, loads in flight too
-        double l[7];
+        for (int q = 0; q < 8; ++q) l[q] = b + q * NG < G ? __ldcg(part + (size_t)(b + q * NG) * kPart + k) : 0.0;
 #pragma unroll
-        for (int q = 0; q < 7; ++q) l[q] = b + q * NG < G ? __ldcg(part + (size_t)(b + q * NG) * kPart + k) : 0.0;
-        t += ((l[0] + l[1]) + (l[2] + l[3])) + ((l[4] + l[5]) + l[6]);
+        for (int q = 0; q < 8; ++q)
+          if (b + q * NG < G) t += l[q];
       }
       s_grp[g * kPart + k] = t;
     }
@@ -268,7 +274,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
     }
     if (!vbar(a.bar, epoch, &s_flag, a.wait_ns)) goto timeout;
     // scalars of column l in lane l of warp 0
-    double sg = 0.0, sden = 0.0, sig_ = 0.0, sthr = 0.0, sbb = 0.0, srr = 0.0, sal = 0.0;
+    double sden = 0.0, sig_ = 0.0, sthr = 0.0, sbb = 0.0, srr = 0.0, sal = 0.0;
     int sact = 0;
     double t = gather_sums();
     if (warp == 0) {
@@ -278,7 +284,6 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
         sbb = bb;
         srr = rr;
         sthr = a.tol * a.tol * bb;
-        sg = g;
         sden = dl;
         sig_ = 1.0 / g;
         sact = (rr <= sthr || !(dl > 0.0)) ? 0 : 1;
@@ -320,17 +325,22 @@ __global__ void __launch_bounds__(MAXT, 1) pcg64_kernel(PcgArgsT<double> a, int 
       if (warp == 0) {
         const double g = t, dl = __shfl_sync(0xffffffffu, t, (lane + 3) & 31),
                      rr = __shfl_sync(0xffffffffu, t, (lane + 6) & 31);
+        const double be = g * sig_;
+        const double den = fma(-be, be * sden, dl);
+        // 1 / den in lanes 0 .. 2 and 1 / g, for the next iteration, in 3 .. 5
+        const double gs = __shfl_sync(0xffffffffu, g, (lane + 29) & 31);
+        const double inv = inv_n(lane < NR ? den : gs);
+        const double al = g * inv, ig = __shfl_sync(0xffffffffu, inv, (lane + NR) & 31);
         if (lane < NR && sact) {
           srr = rr;
-          const double be = g * sig_;
-          const double den = dl - be * be * sden;
-          if (rr <= sthr || !(den > 0.0)) {  // converged, or breakdown: stop this column
-            sact = 0;
+          // rr <= sthr on the bits (both are sums of squares)
+          if (__double_as_longlong(rr) <= __double_as_longlong(sthr) || !positive_n(den)) {
+            sact = 0;  // converged, or breakdown: stop this column
             s_act[lane] = 0;
           } else {
             s_be[lane] = be;
-            s_al[lane] = g / den;
-            sig_ = 1.0 / g;
+            s_al[lane] = al;
+            sig_ = ig;
             sden = den;
           }
         }
@@ -371,7 +381,7 @@ timeout:
 
 namespace {
 size_t pcg64_smem(int rows, bool coarse) {
-  return (size_t)rows * (8 * kEll + 4 * kEll + (coarse ? 8 * kModes : 0));
+  return (size_t)rows * (8 * kEll + 4 * kEll + (coarse ? 8 * kModes + 8 * NR : 0)) + (coarse ? 8 * kModes : 0);
 }
 
 template <int MAXT, bool C>

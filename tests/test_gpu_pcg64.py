@@ -86,8 +86,8 @@ def test_coupling_solve_residual(name):
 # the generic kernel (csrc/emu_pcg64.cu, pcg16_columns), with a full and a
 # ragged last block of 128 rows: a handle's first solve reaches its tolerance.
 SETUPS = {
-    "rows_128": lambda: box_beam(1, 1, 31),
-    "rows_132": lambda: box_beam(1, 1, 32),
+    "rows_128": lambda: box_beam(3, 3, 7),
+    "rows_132": lambda: box_beam(2, 3, 10),
     "two_columns_3k": lambda: mtu_for_tet_count(12000),
     "four_columns_9k": lambda: mtu_for_tet_count(40000),
     "generic_13k": lambda: mtu_for_tet_count(60000),
