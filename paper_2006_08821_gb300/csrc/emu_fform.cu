@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(256) k_rhs_fform(TetArgs<double> a) {
 // g = V P(F) + alpha w (F - G_i q) - nu (Eqs. 6-7, Sec. 3.4), |g|^2; the
 // factor of H = hessian_F + alpha w I and y = H^-1 g.
 __global__ void __launch_bounds__(128) k_grad_fform(TetArgs<double> a) {
+  dep_sync();
   const int64_t m = a.m;
   double acc[1] = {0.0};
   int bad = 0;
@@ -299,6 +300,7 @@ __global__ void __launch_bounds__(128) k_grad_fform(TetArgs<double> a) {
 // 3r .. 3r+2. The block sums -Yh^T Yh (the Woodbury term of Eq. 12) and
 // B y = sum_i w_i (G_i Phi)^T y_i: By[16r+j] = sum_i w_i sum_b y[r][b] gam_j[b].
 __global__ void __launch_bounds__(256) k_syrk_fform(TetArgs<double> a, double* __restrict__ cpart) {
+  dep_sync();
   constexpr int CH = kSyrk64Chunk;  // tets per chunk
   constexpr int KR = CH * 9;
   __shared__ double sY[KR][kK + 1];
@@ -391,6 +393,7 @@ __global__ void __launch_bounds__(256) k_syrk_fform(TetArgs<double> a, double* _
 // ------------------------------------------------------------ direction ---
 // d = -(y + alpha w H^-1 v), v = (G_i Phi) z; g . d; corners of w G^T d.
 __global__ void __launch_bounds__(128) k_dir_fform(TetArgs<double> a) {
+  dep_sync();
   __shared__ double sz[kK];
   for (int k = threadIdx.x; k < kK; k += blockDim.x) sz[k] = a.z[k];
   __syncthreads();
@@ -439,6 +442,7 @@ __global__ void __launch_bounds__(128) k_dir_fform(TetArgs<double> a) {
 // the ACAP part's two coefficients alpha w <D, dD>, alpha w |dD|^2 with
 // D = G q - F, dD = G dq - d.
 __global__ void __launch_bounds__(128) k_ls_fform(TetArgs<double> a, LsSelect sel) {
+  dep_sync();
   const double rho = sel.rho;
   const int64_t m = a.m;
   const double s0 = a.sc->sigma_start;
@@ -516,6 +520,7 @@ __global__ void __launch_bounds__(128) k_ls_fform(TetArgs<double> a, LsSelect se
 
 // ------------------------------------------------------------ update ------
 __global__ void __launch_bounds__(256) k_update_fform(TetArgs<double> a, double* __restrict__ q) {
+  dep_sync();
   const double sig = a.sc->sigma;
   if (sig == 0.0) return;
   const int64_t m = a.m;
@@ -585,19 +590,19 @@ static int fform_grid(int64_t m, int threads) { return (int)(m > 0 ? (m + thread
 
 void launch_rhs_fform(const TetArgs<double>& a, int grid, cudaStream_t st) { k_rhs_fform<<<grid, 256, 0, st>>>(a); }
 void launch_grad_fform(const TetArgs<double>& a, int grid, int threads, cudaStream_t st) {
-  k_grad_fform<<<grid, threads, 0, st>>>(a);
+  launch_dep(a.m <= kDepTets, k_grad_fform, grid, threads, 0, st, a);
 }
 void launch_syrk_fform(const TetArgs<double>& a, int grid, double* cpart, cudaStream_t st) {
-  k_syrk_fform<<<grid, 256, 0, st>>>(a, cpart);
+  launch_dep(a.m <= kDepTets, k_syrk_fform, grid, 256, 0, st, a, cpart);
 }
 void launch_dir_fform(const TetArgs<double>& a, int grid, int threads, cudaStream_t st) {
-  k_dir_fform<<<grid, threads, 0, st>>>(a);
+  launch_dep(a.m <= kDepTets, k_dir_fform, grid, threads, 0, st, a);
 }
 void launch_ls_fform(const TetArgs<double>& a, int grid, int threads, const LsSelect& sel, cudaStream_t st) {
-  k_ls_fform<<<grid, threads, 0, st>>>(a, sel);
+  launch_dep(a.m <= kDepTets, k_ls_fform, grid, threads, 0, st, a, sel);
 }
 void launch_update_fform(const TetArgs<double>& a, int grid, double* q, cudaStream_t st) {
-  k_update_fform<<<grid, 256, 0, st>>>(a, q);
+  launch_dep(a.m <= kDepTets, k_update_fform, grid, 256, 0, st, a, q);
 }
 void launch_fform_to_Rs(int64_t m, const double* F, double* R, double* s, cudaStream_t st) {
   k_fform_to_Rs<<<fform_grid(m, 128), 128, 0, st>>>(m, F, R, s);

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(128) k_assemble(int64_t n, const int32_t* __re
                                                   const double* __restrict__ contrib, const double* __restrict__ bfix,
                                                   const uint8_t* __restrict__ is_fixed,
                                                   const double* __restrict__ qfix, int mode, double* __restrict__ b) {
+  dep_sync();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = i / 3;
     double s = 0.0;
@@ -66,7 +67,7 @@ void launch_assemble(int64_t n, const int32_t* slot_ptr, const int32_t* slot_idx
                      const double* bfix, const uint8_t* is_fixed, const double* qfix, int mode, double* b,
                      cudaStream_t st) {
   const int64_t grid = (3 * n + 127) / 128;
-  k_assemble<<<(int)(grid < 1 ? 1 : grid), 128, 0, st>>>(n, slot_ptr, slot_idx, contrib, bfix, is_fixed, qfix, mode, b);
+  launch_dep(n <= kDepTets / 2, k_assemble, (int)(grid < 1 ? 1 : grid), 128, 0, st, n, slot_ptr, slot_idx, contrib, bfix, is_fixed, qfix, mode, b);
 }
 
 // ------------------------------------------------------------ gradient ----
@@ -74,6 +75,7 @@ void launch_assemble(int64_t n, const int32_t* slot_ptr, const int32_t* slot_idx
 // Uw and y = H_F^-1 g = (g - N g) / (alpha w) in TW.
 template <typename TW>
 __global__ void __launch_bounds__(128) k_grad(TetArgs<TW> a) {
+  dep_sync();
   const int64_t m = a.m;
   double acc[1] = {0.0};
   int bad = 0;
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(128) k_grad(TetArgs<TW> a) {
 }
 
 template <typename TW> void launch_grad(const TetArgs<TW>& a, int grid, int threads, cudaStream_t st) {
-  k_grad<TW><<<grid, threads, 0, st>>>(a);
+  launch_dep(a.m <= kDepTets, k_grad<TW>, grid, threads, 0, st, a);
 }
 
 // ------------------------------------------------------------ capacitance --
@@ -149,6 +151,7 @@ template <typename TW> void launch_grad(const TetArgs<TW>& a, int grid, int thre
 // Also B y = sum_i w_i (G_i Phi^T)^T y_i: By[16r+j] = sum_i w_i sum_b y[r][b] gam_j[b].
 template <typename TW>
 __global__ void __launch_bounds__(256) k_syrk(TetArgs<TW> a, double* __restrict__ cpart) {
+  dep_sync();
   // tets per chunk: few in FP64, whose pipe takes 10 us per 8 tets, so that
   // the chunks of a small mesh spread evenly over the SMs (6,080 tets at two
   // blocks per SM: 10 chunks of 4 on every SM, before 48 or 24 tets)
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(256) k_syrk(TetArgs<TW> a, double* __restrict_
 }
 
 template <typename TW> void launch_syrk(const TetArgs<TW>& a, int grid, double* cpart, cudaStream_t st) {
-  k_syrk<TW><<<grid, 256, 0, st>>>(a, cpart);
+  launch_dep(a.m <= kDepTets, k_syrk<TW>, grid, 256, 0, st, a, cpart);
 }
 
 // ------------------------------------------- capacitance sum and solve ----
@@ -274,6 +277,7 @@ constexpr int kCapOwn = (kCapSums + 255) / 256;   // entries a thread of the sol
 template <typename T>
 __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, int nblk, double* __restrict__ cfull,
                                              const double* __restrict__ cadd, double* z, DevScalars* sc) {
+  dep_sync();
   const int tid = threadIdx.x, lane = tid & 31;
   {
     const int e = blockIdx.x * 8 + (tid >> 5);
@@ -446,15 +450,16 @@ void launch_cap_solve(const double* cpart, int nblk, const double* cfull_scratch
   double* cfull = const_cast<double*>(cfull_scratch);
   const int grid = (kCapSums + 7) / 8;
   if (fp32_factor)
-    k_cap<float><<<grid, 256, 0, st>>>(cpart, nblk, cfull, cadd, z, sc);
+    launch_dep(nblk <= kDepTets / 32, k_cap<float>, grid, 256, 0, st, cpart, nblk, cfull, cadd, z, sc);
   else
-    k_cap<double><<<grid, 256, 0, st>>>(cpart, nblk, cfull, cadd, z, sc);
+    launch_dep(nblk <= kDepTets / 32, k_cap<double>, grid, 256, 0, st, cpart, nblk, cfull, cadd, z, sc);
 }
 
 // ------------------------------------------------------------ direction ---
 // d = -(y + alpha H_F^-1 w (G Phi^T) z) = -(y + (I - N) v), v = (G_i Phi^T) z.
 template <typename TW>
 __global__ void __launch_bounds__(128) k_dir(TetArgs<TW> a) {
+  dep_sync();
   __shared__ double sz[kK];
   for (int k = threadIdx.x; k < kK; k += blockDim.x) sz[k] = a.z[k];
   __syncthreads();
@@ -511,7 +516,7 @@ __global__ void __launch_bounds__(128) k_dir(TetArgs<TW> a) {
 }
 
 template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, int threads, cudaStream_t st) {
-  k_dir<TW><<<grid, threads, 0, st>>>(a);
+  launch_dep(a.m <= kDepTets, k_dir<TW>, grid, threads, 0, st, a);
 }
 
 // ------------------------------------------------------------ line search --
@@ -522,6 +527,7 @@ template <typename TW> void launch_dir(const TetArgs<TW>& a, int grid, int threa
 // alpha/2 sum w |D + sigma dD|^2 - |D|^2, D = G q - F, dD = G dq - d.
 template <typename TW>
 __global__ void __launch_bounds__(128) k_ls(TetArgs<TW> a, LsSelect sel) {
+  dep_sync();
   const double rho = sel.rho;
   const int64_t m = a.m;
   const double s0 = a.sc->sigma_start;
@@ -608,7 +614,7 @@ __global__ void __launch_bounds__(128) k_ls(TetArgs<TW> a, LsSelect sel) {
 }
 
 template <typename TW> void launch_ls(const TetArgs<TW>& a, int grid, int threads, const LsSelect& sel, cudaStream_t st) {
-  k_ls<TW><<<grid, threads, 0, st>>>(a, sel);
+  launch_dep(a.m <= kDepTets, k_ls<TW>, grid, threads, 0, st, a, sel);
 }
 
 // ------------------------------------------------------------ update ------
@@ -616,6 +622,7 @@ template <typename TW> void launch_ls(const TetArgs<TW>& a, int grid, int thread
 // polar factor Rx is close to I; R' = R Rx, S' = sym(Rx^T X).
 template <typename TW>
 __global__ void __launch_bounds__(128) k_update_tets(TetArgs<TW> a, double* __restrict__ q) {
+  dep_sync();
   const double sig = a.sc->sigma;
   if (sig == 0.0) return;
   const int64_t m = a.m;
@@ -645,7 +652,7 @@ __global__ void __launch_bounds__(128) k_update_tets(TetArgs<TW> a, double* __re
 }
 
 template <typename TW> void launch_update_tets(const TetArgs<TW>& a, int grid, int threads, double* q, cudaStream_t st) {
-  k_update_tets<TW><<<grid, threads, 0, st>>>(a, q);
+  launch_dep(a.m <= kDepTets, k_update_tets<TW>, grid, threads, 0, st, a, q);
 }
 
 // ------------------------------------------------------------ normaliser --

@@ -111,6 +111,7 @@ __device__ __forceinline__ void corners_f(TO* __restrict__ contrib, int64_t i, f
 
 // ------------------------------------------------------------ gradient ----
 __global__ void __launch_bounds__(128, 4) k_grad_m(MixArgs a) {
+  dep_sync();
   const int64_t m = a.m;
   // per-thread sums in FP32 (a few tets each), FP64 from the block sum on:
   // GB300's FP64 pipe issues far below its FP32 rate, and per-tet FP64
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(128, 4) k_grad_m(MixArgs a) {
   grad_finish(a.sc, a.partials);
 }
 
-void launch_grad_mixed(const MixArgs& a, int grid, cudaStream_t st) { k_grad_m<<<grid, 128, 0, st>>>(a); }
+void launch_grad_mixed(const MixArgs& a, int grid, cudaStream_t st) { launch_dep(a.m <= kDepTets, k_grad_m, grid, 128, 0, st, a); }
 
 // ------------------------------------------------------------ capacitance --
 // C = sum_i Yh_i^T Yh_i with Yh_i = sqrt(w_i) U_i (G_i Phi^T) (6 x 48 per
@@ -219,6 +220,7 @@ constexpr size_t kTcSmem = kTcYBytes + 2 * kTcRawBytes;
 
 template <bool VEC>
 __global__ void __launch_bounds__(256, kTcBlocksPerSM) k_syrk_tc(MixArgs a, double* __restrict__ cpart) {
+  dep_sync();
   constexpr int CH = kTcCH, LD = kTcLD, RL = kTcRL;
   __shared__ const float* s_src[kTcRawRows];  // first element of each raw row
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -402,9 +404,9 @@ cudaError_t prepare_syrk_tc() {
 
 void launch_syrk_tc(const MixArgs& a, int grid, double* cpart, cudaStream_t st) {
   if (a.m % 4 == 0)
-    k_syrk_tc<true><<<grid, 256, kTcSmem, st>>>(a, cpart);
+    launch_dep(a.m <= kDepTets, k_syrk_tc<true>, grid, 256, kTcSmem, st, a, cpart);
   else
-    k_syrk_tc<false><<<grid, 256, kTcSmem, st>>>(a, cpart);
+    launch_dep(a.m <= kDepTets, k_syrk_tc<false>, grid, 256, kTcSmem, st, a, cpart);
 }
 
 // ------------------------------------------------------------ direction ---
@@ -412,6 +414,7 @@ void launch_syrk_tc(const MixArgs& a, int grid, double* cpart, cudaStream_t st) 
 // registers, so more tets are in flight per SM; the second pass is served
 // mostly by L1.
 __global__ void __launch_bounds__(128, 8) k_dir_m(MixArgs a) {
+  dep_sync();
   __shared__ float sz[kK];
   if (threadIdx.x < kK) sz[threadIdx.x] = (float)a.z[threadIdx.x];
   __syncthreads();
@@ -483,7 +486,7 @@ __global__ void __launch_bounds__(128, 8) k_dir_m(MixArgs a) {
   block_reduce_write<1>(acc, a.partials + blockIdx.x);
 }
 
-void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st) { k_dir_m<<<grid, 128, 0, st>>>(a); }
+void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st) { launch_dep(a.m <= kDepTets, k_dir_m, grid, 128, 0, st, a); }
 
 // ------------------------------------------------------------ line search --
 // V [Psi(F + s d) - Psi(F)] with M = F^-1 d = S^-1 R^T d and
@@ -492,6 +495,7 @@ void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st) { k_dir_m<<<g
 //   + lam/2 log1p(x) (2 ln J + log1p(x)) + ka (2 s (Fu).(du) + s^2 |du|^2),
 // with F - F^-T = R (2E + E^2) S^-1; plus the ACAP coefficients.
 __global__ void __launch_bounds__(128) k_ls_m(MixArgs a, LsSelect sel) {
+  dep_sync();
   const float rho = (float)sel.rho;
   const int64_t m = a.m;
   const float s0 = (float)a.sc->sigma_start;
@@ -578,7 +582,7 @@ __global__ void __launch_bounds__(128) k_ls_m(MixArgs a, LsSelect sel) {
 }
 
 void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream_t st) {
-  k_ls_m<<<grid, 128, 0, st>>>(a, sel);
+  launch_dep(a.m <= kDepTets, k_ls_m, grid, 128, 0, st, a, sel);
 }
 
 // ------------------------------------------------------------ update ------
@@ -590,6 +594,7 @@ void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream
 // changes none of them).
 __global__ void __launch_bounds__(128) k_update_m(MixArgs a, double* __restrict__ q, const double* __restrict__ dq64,
                                                   float* __restrict__ uh, float* __restrict__ ul) {
+  dep_sync();
   const double sigd = a.sc->sigma;
   if (sigd == 0.0) return;
   const float sig = (float)sigd;
@@ -624,7 +629,7 @@ __global__ void __launch_bounds__(128) k_update_m(MixArgs a, double* __restrict_
 
 void launch_update_mixed(const MixArgs& a, int grid, double* q, const double* dq64, float* uh, float* ul,
                          cudaStream_t st) {
-  k_update_m<<<grid, 128, 0, st>>>(a, q, dq64, uh, ul);
+  launch_dep(a.m <= kDepTets, k_update_m, grid, 128, 0, st, a, q, dq64, uh, ul);
 }
 
 __global__ void __launch_bounds__(256) k_split_disp(int64_t n3, const double* __restrict__ q, const double* __restrict__ Q,
@@ -711,6 +716,7 @@ __global__ void __launch_bounds__(128) k_assemble_f(int64_t n, const int32_t* __
                                                     const int32_t* __restrict__ slot_idx,
                                                     const float* __restrict__ contrib,
                                                     const uint8_t* __restrict__ is_fixed, float* __restrict__ b) {
+  dep_sync();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = i / 3;
     b[i] = is_fixed[v] ? 0.f : gather_corners(slot_idx, slot_ptr[v], slot_ptr[v + 1], contrib + (i - 3 * v));
@@ -720,7 +726,7 @@ __global__ void __launch_bounds__(128) k_assemble_f(int64_t n, const int32_t* __
 void launch_assemble_f(int64_t n, const int32_t* slot_ptr, const int32_t* slot_idx, const float* contrib,
                        const uint8_t* is_fixed, float* b, cudaStream_t st) {
   const int64_t grid = (3 * n + 127) / 128;
-  k_assemble_f<<<(int)(grid < 1 ? 1 : grid), 128, 0, st>>>(n, slot_ptr, slot_idx, contrib, is_fixed, b);
+  launch_dep(n <= kDepTets / 2, k_assemble_f, (int)(grid < 1 ? 1 : grid), 128, 0, st, n, slot_ptr, slot_idx, contrib, is_fixed, b);
 }
 
 // ------------------------------------------------------------ conversion --

@@ -196,6 +196,7 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 
 __global__ void __launch_bounds__(kThreads, kSyrk05BlocksPerSM)
     k_syrk05(MixArgs a, double* __restrict__ cpart, const __grid_constant__ Syrk05Maps maps) {
+  dep_sync();
   extern __shared__ __align__(16) unsigned char smem_dyn[];
   __shared__ __align__(8) uint64_t bar_full[kStages], bar_mma[kTiles];
   __shared__ uint32_t s_taddr;
@@ -422,7 +423,7 @@ bool make_syrk05_maps(const MixArgs& a, Syrk05Maps* maps) {
 }
 
 void launch_syrk05(const MixArgs& a, const Syrk05Maps& maps, int grid, double* cpart, cudaStream_t st) {
-  k_syrk05<<<grid, kThreads, kSmemBytes, st>>>(a, cpart, maps);
+  launch_dep(a.m <= kDepTets, k_syrk05, grid, kThreads, kSmemBytes, st, a, cpart, maps);
 }
 
 }  // namespace emu
