@@ -135,15 +135,15 @@ def algorithmic_bytes(phase, mixed, m, n, nnz, cg_iters, fform=False):
     return None
 
 
-# per-tet kernels launched per launch of a profiled phase (the update phase
-# also launches the per-vertex position update, the mixed gradient phase the
-# per-vertex split of the displacement)
-PER_TET_KERNELS = {"grad": 0.5, "syrk": 1.0, "dir": 1.0, "ls": 1.0, "update": 0.5}
-PER_TET_KERNELS_FP64 = {"grad": 1.0, "syrk": 1.0, "dir": 1.0, "ls": 1.0, "update": 0.5}
+# phases with one per-tet kernel per launch
+PER_TET_KERNELS = ("grad", "syrk", "dir", "ls", "update")
 
 
-def per_tet_kernels(mixed):
-    return PER_TET_KERNELS if mixed else PER_TET_KERNELS_FP64
+def per_tet_launches(prof, name):
+    """Per-tet kernel launches of a profiled phase: all of them, except that the
+    update's runs once per capacitance product (a Newton iteration)."""
+    nl = prof.get(name, (0.0, 0))[1]
+    return prof.get("syrk", (0.0, 0))[1] or nl if name == "update" else nl
 
 
 def per_tet_fractions(prof, mixed, m, n, nnz, peak, traffic_table=None, fform=False):
@@ -151,11 +151,11 @@ def per_tet_fractions(prof, mixed, m, n, nnz, peak, traffic_table=None, fform=Fa
     CUDA-event duration, against the HBM peak; with the kernel's ncu DRAM
     bytes per launch beside it where a capture of the unchanged kernel exists."""
     out = {}
-    for name, per in per_tet_kernels(mixed).items():
+    for name in PER_TET_KERNELS:
         ms, nl = prof.get(name, (0.0, 0))
         if nl <= 0 or ms <= 0:
             continue
-        launches = nl * per
+        launches = per_tet_launches(prof, name)
         b = algorithmic_bytes(name, mixed, m, n, nnz, 0.0, fform)
         us = 1e3 * ms / launches
         gbs = b / (us * 1e-6) / 1e9
@@ -219,9 +219,8 @@ def whole_iteration(prof, mixed, m, n, nnz, cg_total, iters, peak, value, fform=
     if iters <= 0:
         return None
     b = 0.0
-    for name, per in per_tet_kernels(mixed).items():
-        ms, nl = prof.get(name, (0.0, 0))
-        b += algorithmic_bytes(name, mixed, m, n, nnz, 0.0, fform) * nl * per
+    for name in PER_TET_KERNELS:
+        b += algorithmic_bytes(name, mixed, m, n, nnz, 0.0, fform) * per_tet_launches(prof, name)
     b += algorithmic_bytes("pcg", mixed, m, n, nnz, cg_total)
     b /= iters
     t = sum(v[0] for v in prof.values()) / 1e3 / iters

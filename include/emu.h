@@ -196,7 +196,8 @@ typedef struct {
  *                   the fastest: the local polynomial's degree (2, 3, 4, 6,
  *                   8; overrides cg_local_degree) for the mixed path's dq
  *                   solves, and the rows per block (64, 128, 256) of the
- *                   FP64 CG. Each choice is kept for the process per device
+ *                   FP64 CG's generic kernel (systems above 320 rows per
+ *                   SM; smaller ones have one shape). Each choice is kept for the process per device
  *                   and mesh size, so handles of one mesh run the same
  *                   settings; another process may choose differently, and
  *                   its results then differ in rounding. emu_get_tuning
@@ -406,7 +407,7 @@ int emu_eval_stretch_terms(const double* s, const double* params, int64_t n, int
 
 /* Launch settings of the coupling solves in use: the local polynomial's
  * degree of the mixed path's pipelined CG (0 where that CG is not used),
- * the rows per block of the FP64 CG, and whether emu_create ran the
+ * the rows per block of the FP64 CG's generic kernel, and whether emu_create ran the
  * autotuner. Any pointer may be NULL. */
 int emu_get_tuning(emu_handle* h, int32_t* cg_local_degree, int32_t* cg64_rows_per_block, int32_t* tuned);
 

@@ -105,22 +105,25 @@ __global__ void __launch_bounds__(128) k_bone_eval(BoneArgs a, double* gref_out)
   __shared__ double sy[kMaxFreeBones][9];    // w_b y_b
   __shared__ double sg2[kMaxFreeBones];
   __shared__ double sYh[kMaxFreeBones][6][kK];
+  __shared__ double sA[kMaxFreeBones * 9];   // sum c_i (G_i q - I)
   __shared__ int sbad;
   const int tid = threadIdx.x;
   if (tid == 0) sbad = 0;
+  if (tid < a.nfb * 9) {  // one entry per thread (one thread's 288 FP64 additions took 10 us)
+    const double* p = a.part + (size_t)(tid / 9) * kBoneMeanBlocks * 9 + tid % 9;
+    double t = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < kBoneMeanBlocks; ++k) t += p[9 * k];
+    sA[tid] = t;
+  }
   __syncthreads();
   const bool gref = gref_out != nullptr;
   if (tid < a.nfb) {
     const int b = tid;
-    const double ct = a.alpha * a.wb[b];
+    const double ct = a.alpha * a.wb[b], ict = inv_n(ct);
     double AmI[9];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) AmI[e] = 0.0;
-    for (int k = 0; k < kBoneMeanBlocks; ++k)
-#pragma unroll
-      for (int e = 0; e < 9; ++e) AmI[e] += a.part[((size_t)b * kBoneMeanBlocks + k) * 9 + e];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) AmI[e] /= ct;
+    for (int e = 0; e < 9; ++e) AmI[e] = sA[9 * b + e] * ict;
     double R[9], RmI[9], S[9], E[9], RE[9], Dm[9];
     bone_state(a, b, gref, R, RmI, S, E);
     matmul3(R, E, RE);
@@ -159,7 +162,7 @@ __global__ void __launch_bounds__(128) k_bone_eval(BoneArgs a, double* gref_out)
       const double sw = sqrt(a.wb[b]);
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        y[k] /= ct;
+        y[k] *= ict;
         o[kBoneG + k] = g[k];
         o[kBoneY + k] = y[k];
         sy[b][k] = a.wb[b] * y[k];
@@ -197,6 +200,7 @@ __global__ void __launch_bounds__(128) k_bone_eval(BoneArgs a, double* gref_out)
   __syncthreads();
   for (int e = tid; e < kK * kK; e += blockDim.x) {
     const int row = e / kK, col = e % kK;
+    if (col > row) continue;  // the capacitance kernel adds the lower triangle
     double acc = a.cconst[e];
     for (int b = 0; b < a.nfb; ++b)
 #pragma unroll
@@ -215,30 +219,31 @@ __global__ void __launch_bounds__(128) k_bone_eval(BoneArgs a, double* gref_out)
 }
 
 // ------------------------------------------------------------ bone dir ----
-__global__ void k_bone_dir(BoneArgs a, const double* __restrict__ z, double* gtd_out) {
+// One warp per free bone, an entry of F per lane (one thread took 280 FP64
+// instructions, 12.7 us).
+__global__ void __launch_bounds__(32 * kMaxFreeBones) k_bone_dir(BoneArgs a, const double* __restrict__ z, double* gtd_out) {
   __shared__ double sgtd[kMaxFreeBones];
-  const int b = threadIdx.x;
+  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (b < a.nfb) {
     double* o = a.bst + (size_t)b * kBoneStride;
     const double* gb = a.gbar + (size_t)b * kK;
-    double v[9];
+    const int e = lane < 9 ? lane : 0, k6 = lane < 6 ? lane : 0;
+    double v = 0.0;
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int j = 0; j < 16; ++j) v += z[16 * (e / 3) + j] * gb[3 * j + e % 3];
+    // (I - N) v with N = U^T U
+    double t = 0.0, x = 0.0;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        double x = 0.0;
-        for (int j = 0; j < 16; ++j) x += z[16 * r + j] * gb[3 * j + c];
-        v[3 * r + c] = x;
-      }
-    apply_I_minus_N(o + kBoneU, v);
+    for (int j = 0; j < 9; ++j) t += o[kBoneU + 9 * k6 + j] * __shfl_sync(0xffffffffu, v, j);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) x += o[kBoneU + 9 * k + e] * __shfl_sync(0xffffffffu, t, k);
+    const double d = -(o[kBoneY + e] + (v - x));
+    const double gd = o[kBoneG + e] * d;
+    if (lane < 9) o[kBoneD + e] = d;
     double gtd = 0.0;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const double d = -(o[kBoneY + k] + v[k]);
-      o[kBoneD + k] = d;
-      gtd += o[kBoneG + k] * d;
-    }
-    sgtd[b] = gtd;
+    for (int k = 0; k < 9; ++k) gtd += __shfl_sync(0xffffffffu, gd, k);
+    if (lane == 0) sgtd[b] = gtd;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -650,7 +655,7 @@ void launch_bone_eval(const BoneArgs& a, double* gref_out, cudaStream_t st) {
 }
 
 void launch_bone_dir(const BoneArgs& a, const double* z, double* gtd_out, cudaStream_t st) {
-  k_bone_dir<<<1, 32, 0, st>>>(a, z, gtd_out);
+  k_bone_dir<<<1, 32 * (a.nfb > 0 ? a.nfb : 1), 0, st>>>(a, z, gtd_out);
 }
 
 void launch_bone_ls(const BoneArgs& a, const float* dq32, double rho, double* partials_out, cudaStream_t st) {

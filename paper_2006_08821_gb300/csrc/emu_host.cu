@@ -1290,7 +1290,13 @@ int emu_set_external_forces(emu_handle* h, const double* f, int64_t n_verts) {
     EMU_CK(cudaMemcpyAsync(h->sc, &init, sizeof(init), cudaMemcpyHostToDevice, h->st));
     EMU_CK(cudaMemcpyAsync(rhs, fb.data(), 24 * n, cudaMemcpyHostToDevice, h->st));
     EMU_CK(cudaMemsetAsync(x, 0, 24 * n, h->st));
-    EMU_CK(launch_pcg<double>(3, h->pcg64(rhs, x, 1e-13), h->grid_pcg3, h->st));
+    PcgArgsT<double> pa = h->pcg64(rhs, x, 1e-13);
+    // Mixed path: the generic kernel (it is the one without phit). A last-bit
+    // change of nu moves its FP32 copy here and there, and a cantilever's
+    // converged positions by up to 1e-5 of the mesh at 1e-6 (soft bending
+    // modes), so a one-off solve is no place to change the rounding.
+    if (h->mixed) pa.phit = nullptr;
+    EMU_CK(launch_pcg<double>(3, pa, h->grid_pcg3, h->st));
     launch_nu(m, h->tet, h->Dinv, h->w, x, h->nu64, h->mixed ? h->nu32 : nullptr, h->st);
     EMU_CK(cudaGetLastError());
     DevScalars out;
@@ -1366,16 +1372,20 @@ namespace {
 // (split: form the displacement's float pair from q first; the update kernel
 // has left it when q was only advanced by a step since)
 int enqueue_grad(emu_handle* h, bool split) {
+  if (h->mixed && split) {
+    h->ph_begin();
+    launch_split_disp(h->n, h->q, h->Qrest, h->uh32, h->ul32, h->st);
+    h->ph_end(EMU_PHASE_ASSEMBLE, 1);
+  }
   h->ph_begin();
   if (h->mixed) {
-    if (split) launch_split_disp(h->n, h->q, h->Qrest, h->uh32, h->ul32, h->st);
     launch_grad_mixed(h->margs(), h->grid_tet4, h->st);
   } else if (h->fform) {
     launch_grad_fform(h->args<double>(), h->grid_t64, h->threads_t64, h->st);
   } else {
     launch_grad<double>(h->args<double>(), h->grid_t64, h->threads_t64, h->st);
   }
-  h->ph_end(EMU_PHASE_GRAD, h->mixed && split ? 2 : 1);
+  h->ph_end(EMU_PHASE_GRAD, 1);
   if (h->nfb > 0) {  // the free bones' virtual elements (Sec. 3.3)
     h->ph_begin();
     bones_after_grad(h);

@@ -271,9 +271,9 @@ constexpr int kCapOwn = (kCapSums + 255) / 256;   // entries a thread of the sol
 // entries are a prefix and whole warps drop out as it shrinks. In FP64 a warp
 // instruction holds GB300's FP64 pipe for 16 cycles: 9.2e3 cycles for the
 // updates, and the pivots' reciprocals are Newton steps in one warp.
-// Measured per launch pair before (reduction, then a 256-thread factorisation
-// with a barrier and a division per column): FP32 27 us, FP64 95 us a Newton
-// iteration; the fused kernel's figures stand in the kernel table.
+// Measured per Newton iteration with the reduction (phase times): FP32 27 us
+// as two launches with a barrier and a division per column, 19 us now; FP64 83
+// us, 33 us now.
 template <typename T>
 __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, int nblk, double* __restrict__ cfull,
                                              const double* __restrict__ cadd, double* z, DevScalars* sc) {

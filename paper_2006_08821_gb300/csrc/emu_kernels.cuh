@@ -20,10 +20,11 @@ struct LsSelect {
 };
 
 // Launch shape of the FP64 per-tet kernels. A warp instruction holds an SM's
-// FP64 pipe for 16 cycles, so a mesh that fits in one warp per block is
-// spread one warp at a time over the SMs (128-thread blocks left 140 of 152
-// SMs idle on a 1,536-tet beam: gradient 69, direction 18, line search 29,
-// update 27 us). From 8 warps per SM on (m > 256 per SM) every SM is busy
+// FP64 pipe for 19 cycles and its own warp for 64, so a mesh that fits in one
+// warp per block is spread one warp at a time over the SMs (128-thread blocks
+// left 140 of 152 SMs idle on a 1,536-tet beam; update and position update 27
+// -> 23 us, the others stay bound by one warp's instruction count). From 8
+// warps per SM on (m > 256 per SM) every SM is busy
 // either way and 128-thread blocks keep the partial sums few.
 inline void tet64_shape(int64_t m, int sms, int* grid, int* threads) {
   *threads = m <= 256 * (int64_t)sms ? 32 : 128;

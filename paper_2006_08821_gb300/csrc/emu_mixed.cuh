@@ -58,7 +58,7 @@ void launch_grad_mixed(const MixArgs& a, int grid, cudaStream_t st);
 void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st);
 // Line-search constants and the direction kernel's g.d partials, for the
 // Trial energies of one pass and, in its last block, the selected step
-// (k_ls_select's work); the gradient kernel likewise leaves ||g||^2 in sc.
+// (ls_finish); the gradient kernel likewise leaves ||g||^2 in sc.
 void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream_t st);
 void launch_update_mixed(const MixArgs& a, int grid, double* q, const double* dq64, float* uh, float* ul,
                          cudaStream_t st);

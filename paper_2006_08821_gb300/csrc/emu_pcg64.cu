@@ -25,10 +25,14 @@
 //     the last block to leave zeroes, so no memset precedes a launch;
 //   * one division on the path from the sums to alpha: with den the last
 //     denominator, beta g / alpha = beta^2 den.
-// Measured on one GB300 against the generic kernel (whole calls): coupling
-// solve of 19,833 rows 4.87 -> 2.08 ms; two-bone arm of 692 rows (45 CG
-// iterations per Newton iteration) 434 -> 226 ms a solve; box beam of 425 rows
-// in FP64 94 -> 72 ms; 6,080-tet unit in FP64 82 -> 67 ms.
+//   * a lane sums one mode of Phi'^T w over half of its warp's rows (17 FP64
+//     instructions; 16 products and a butterfly are 32), products run in one
+//     chain and one reciprocal serves alpha and the next beta: an FP64
+//     instruction holds its warp 64 cycles whatever its lanes or its
+//     neighbours do, so a warp's instruction count is its time.
+// Measured on one GB300 against the generic kernel: coupling solve of 19,833
+// rows 4.83 -> 1.74 ms; an iteration at 425 rows 28 -> 6.8 us, at 692 rows (the
+// arm's 45 an iteration of Newton) 23 -> 7.5 us, at 1,485 rows 28 -> 8.5 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
