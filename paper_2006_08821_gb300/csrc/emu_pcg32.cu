@@ -37,9 +37,9 @@ constexpr int kGather = 16;  // entries of a matrix row gathered at once
 // Entries gathered at once, from the pruned system and from the local table:
 // 8 where the local rows hold at most 8 (a regular grid's pruned rows hold 7),
 // 16 for the rows of an irregular mesh (about 14), whose entries beyond the
-// eighth used to run one dependent load at a time (59,840 tets: 9,400 against
-// 4,300 cycles for the local products and 4,000 against 2,600 for the SpMV of
-// a CG iteration).
+// eighth used to run one dependent load at a time (59,840 tets: 4,000 -> 2,900
+// cycles for the SpMV of a CG iteration; the local products, 9,300 cycles, are
+// bound by shared-memory bank conflicts of the 16-byte gathers either way).
 constexpr int kWideRows = 16, kNarrowRows = 8;
 constexpr int kMaxGridStrides = 8;  // grid_sum_f handles up to 256 blocks
 // words of Pcg32Work::sync, one 128-byte line apart
@@ -64,6 +64,11 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 __device__ __forceinline__ bool gbar(const Pcg32Work& wk, unsigned& epoch, int* s_flag, unsigned long long wait_ns) {
   __syncthreads();
   if (gridDim.x == 1) return true;  // one block: its own barrier is all there is
+  if (wk.cluster) {  // the blocks are one cluster: its hardware barrier orders their global writes too
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  }
   epoch += 1u;
   if (threadIdx.x == 0) {
     red_release_add(wk.sync + kSyncCount, 1u);
@@ -96,6 +101,7 @@ __device__ __forceinline__ bool gbar(const Pcg32Work& wk, unsigned& epoch, int* 
 
 // Kernel exit of every block: the last one out zeroes the barrier words.
 __device__ __forceinline__ void gbar_exit(const Pcg32Work& wk) {
+  if (wk.cluster) return;  // the counters were not used
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -213,7 +219,8 @@ __device__ __forceinline__ void grid_sum_f(const float* __restrict__ part, int n
 // entries stay in registers for the whole launch: every grid barrier ends in
 // an acquire, which empties L1, so rereading them cost two L2 round trips
 // before the gather itself could start (2,000 of 14,500 cycles of a CG
-// iteration on the 6,080-tet unit, 1,100 with the entries held).
+// iteration on the 6,080-tet unit, 1,400 with the entries held; 2,600 of 18,500
+// on the 401,920-tet unit, 1,740 held).
 template <int RPT, int GW, bool HOLD>
 struct MatRows {
   const int32_t* rowptr;
@@ -1073,6 +1080,31 @@ __global__ void k_aphi32(int64_t n, const int32_t* __restrict__ rowptr, const in
 }
 
 namespace {
+// Launch of a CG kernel whose blocks wait on one another. Two to eight blocks
+// (up to 4,096 rows, about 18,000 tets) form one thread-block cluster, which the
+// hardware places together: its barrier takes the place of the polled counter
+// (6,080 tets on three blocks: 55.6 -> 52.8 us of CG per Newton iteration; 16
+// beams together 24.8 -> 24.0 ms). Larger grids are cooperative launches.
+constexpr int kMaxCluster = 8;  // the portable size
+cudaError_t launch_blocks(const void* kernel, int grid, PcgArgsT<float>& a, Pcg32Work& w, size_t smem, cudaStream_t st) {
+  void* params[] = {(void*)&a, (void*)&w};
+  w.cluster = grid >= 2 && grid <= kMaxCluster;
+  if (!w.cluster) return cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(NT), params, smem, st);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = grid;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, kernel, params);
+}
+
 // dynamic shared memory: the coarse rows (C), then on a partitioned system
 // two buffers of the local products and a local table of lw words per row slot
 template <int RPT, bool C>
@@ -1109,8 +1141,7 @@ cudaError_t launch32w(const PcgArgsT<float>& args, const Pcg32Work& work, int gr
   const size_t smem = plain_smem<RPT, C>(parted, lw);
   PcgArgsT<float> a = args;
   Pcg32Work w = work;
-  void* params[] = {(void*)&a, (void*)&w};
-  return cudaLaunchCooperativeKernel((const void*)pcg32_kernel<RPT, C, W>, dim3(grid), dim3(NT), params, smem, st);
+  return launch_blocks((const void*)pcg32_kernel<RPT, C, W>, grid, a, w, smem, st);
 }
 
 template <int RPT, bool C>
@@ -1167,9 +1198,8 @@ cudaError_t launch32p(const PcgArgsT<float>& args, const Pcg32Work& work, int gr
   Pcg32Work w = work;
   const int lw = w.degree > 1 ? w.lw : 0;
   if (lw > cg_local_width_max(RPT) || (w.degree > 1 && !w.loc)) return cudaErrorInvalidValue;
-  void* params[] = {(void*)&a, (void*)&w};
   const void* f = w.lw > kNarrowRows ? (const void*)pcg32p_kernel<RPT, true> : (const void*)pcg32p_kernel<RPT, false>;
-  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(NT), params, pipe_smem<RPT>(lw), st);
+  return launch_blocks(f, grid, a, w, pipe_smem<RPT>(lw), st);
 }
 }  // namespace
 

@@ -84,10 +84,15 @@ def test_coupling_solve_residual(name):
 
 # Set-up of the low-rank basis with one, two and four columns per block and on
 # the generic kernel (csrc/emu_pcg64.cu, pcg16_columns), with a full and a
-# ragged last block of 128 rows: a handle's first solve reaches its tolerance.
+# ragged last block of 128 rows, and the FP32 CG of its solves as one block, as
+# clusters of two and of the largest eight blocks, and as the first cooperative
+# grid above: a handle's first solve reaches its tolerance.
 SETUPS = {
     "rows_128": lambda: box_beam(3, 3, 7),
     "rows_132": lambda: box_beam(2, 3, 10),
+    "two_blocks_817": lambda: mtu_for_tet_count(3000),
+    "eight_blocks_3993": lambda: box_beam(10, 10, 32),
+    "nine_blocks_4114": lambda: box_beam(10, 10, 33),
     "two_columns_3k": lambda: mtu_for_tet_count(12000),
     "four_columns_9k": lambda: mtu_for_tet_count(40000),
     "generic_13k": lambda: mtu_for_tet_count(60000),
