@@ -397,7 +397,8 @@ int solve_dq(emu_handle* h) {
 //    pipelined FP32 CG (its dq solves): one solve to dq_tol from zero per
 //    degree on the right-hand side of a real first Newton direction, the
 //    better of two runs each;
-//  * the rows per block of the FP64 CG (the FP64 path, meshes with bones):
+//  * the rows per block of the FP64 CG's generic kernel (the FP64 path and
+//    meshes with bones, above the sizes of pcg64_kernel):
 //    a fixed count of iterations per candidate on a seeded right-hand side
 //    (the count to a tolerance does not depend on the launch shape).
 // Each candidate runs the same method; only rounding differs between them.

@@ -269,7 +269,7 @@ constexpr int kCapOwn = (kCapSums + 255) / 256;   // entries a thread of the sol
 // barriers per four columns, and the work of the trailing triangle only. The
 // entries are numbered from the last column backwards, so the trailing
 // entries are a prefix and whole warps drop out as it shrinks. In FP64 a warp
-// instruction holds GB300's FP64 pipe for 16 cycles: 9.2e3 cycles for the
+// instruction holds an SM's FP64 pipe for 19 cycles: 1.1e4 cycles for the
 // updates, and the pivots' reciprocals are Newton steps in one warp.
 // Measured per Newton iteration with the reduction (phase times): FP32 27 us
 // as two launches with a barrier and a division per column, 19 us now; FP64 83

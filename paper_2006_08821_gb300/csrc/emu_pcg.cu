@@ -10,6 +10,11 @@
 // result is deterministic. The paper prefactors this matrix with Pardiso
 // (Sec. 3.3); on the GPU an iterative solve with warm starts replaces the
 // sparse back-substitution.
+//
+// This is the generic kernel: any size, columns and precision. Three FP64
+// columns of up to 320 rows per SM and sixteen of up to 64 run the kernels of
+// emu_pcg64.cu (launch_pcg picks; 1.3 to 3 times faster there), the mixed path's
+// FP32 solves those of emu_pcg32.cu.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
