@@ -13,6 +13,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "emu_capslots.h"
 #include "emu_kernels.cuh"
 #include "emu_math.cuh"
 #include "emu_reduce.cuh"
@@ -250,10 +251,8 @@ template <typename TW> void launch_syrk(const TetArgs<TW>& a, int grid, double* 
 __device__ __forceinline__ float pivot_inverse(float d) { return __frcp_rn(d); }
 __device__ __forceinline__ double pivot_inverse(double d) { return inv_n(d); }
 
-constexpr int kCapLow = kK * (kK + 1) / 2;        // entries of the lower triangle
-constexpr int kCapSums = kCapLow + kK;            // and of B y
-constexpr int kCapNB = 4;                         // columns of a panel
-constexpr int kCapOwn = (kCapSums + 255) / 256;   // entries a thread of the solving block owns
+static_assert(kCapN == kK, "emu_capslots.h");
+constexpr int kCapNB = 4;  // columns of a panel
 
 // Sums the per-block partials of C (lower triangle) and B y, one warp per
 // entry (entry-major, coalesced, a fixed shuffle tree), and in the last block
@@ -296,17 +295,9 @@ __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, i
       if (lane == 0) __stcg(cfull + src, cadd ? x + cadd[src] : x);
     }
   }
-  // entry t: column 48 - a and row 48 - b with 0 <= b <= a, t = a (a + 1) / 2 + b (a = 0 is unused)
   int row[kCapOwn], col[kCapOwn];
 #pragma unroll
-  for (int s = 0; s < kCapOwn; ++s) {
-    const int t = 1 + tid + 256 * s;
-    int a = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-    if ((a + 1) * (a + 2) / 2 <= t) ++a;
-    if (a * (a + 1) / 2 > t) --a;
-    col[s] = t <= kCapSums ? kK - a : -1;
-    row[s] = kK - (t - a * (a + 1) / 2);
-  }
+  for (int s = 0; s < kCapOwn; ++s) cap_slot(tid, s, &row[s], &col[s]);
   if (!last_block(&sc->ticket[kTicketCap])) return;
   // In FP64 B y is row 48 of the factorisation, which leaves D^-1 L^-1 (B y)
   // there. In FP32 the third warp substitutes with 1 / sqrt(d) scaling while
@@ -322,12 +313,12 @@ __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, i
   T val[kCapOwn];
 #pragma unroll
   for (int s = 0; s < kCapOwn; ++s) {
-    const int c = col[s] < 0 ? 0 : col[s];
-    const double diag = __ldcg(cfull + c * kK + c);
-    const double v = row[s] < kK ? __ldcg(cfull + row[s] * kK + c) : __ldcg(cfull + kCapEntries + c);
-    val[s] = (T)v;
+    const int c = col[s], src = cap_source(row[s], c);
+    val[s] = T(0);
+    if (src < 0) continue;  // a slot past the last entry
+    val[s] = (T)__ldcg(cfull + src);
     // unused modes (k_modes < 48) have zero rows: identity rows with a zero right-hand side
-    if (diag == 0.0) val[s] = row[s] == c ? T(1) : row[s] == kK ? T(0) : val[s];
+    if (__ldcg(cfull + c * kK + c) == 0.0) val[s] = row[s] == c ? T(1) : row[s] == kK ? T(0) : val[s];
   }
   if (tid == 0) s_ok = 1;
   T x0 = T(0), x1 = T(0);  // FP32: right-hand side rows lane and 32 + lane of the third warp
