@@ -46,8 +46,7 @@ __device__ void sym3_eig(const double* A, double* lam, double* W) {
       const int p = e == 2 ? 1 : 0, q = e == 0 ? 1 : 2, o = 3 - p - q;
       const double apq = a[p][q];
       if (apq == 0.0) continue;
-      const double theta = (a[q][q] - a[p][p]) * inv_n(2.0 * apq);
-      const double ta = inv_n(fabs(theta) + sqrt_n(theta * theta + 1.0)), t = copysign(ta, theta);
+      const double t = jacobi_tan(a[p][p], a[q][q], apq);
       const double c = rsqrt_n(t * t + 1.0), s = t * c;
       const double aop = a[o][p], aoq = a[o][q];
       a[o][p] = a[p][o] = c * aop - s * aoq;

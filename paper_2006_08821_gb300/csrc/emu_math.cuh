@@ -52,6 +52,15 @@ EMU_HD double inv_n(double x) {
 #endif
   return 1.0 / x;
 }
+// a / b. The product with a reciprocal rounds twice (within 1.6 ulps), and the
+// reciprocal of a small subnormal overflows (0 / 1e-310 is 0, not 0 inf), so
+// outside inv_n's range the plain quotient.
+EMU_HD double div_n(double a, double b) {
+#ifdef __CUDA_ARCH__
+  if (mid_range(fabs(b))) return a * inv_n(b);
+#endif
+  return a / b;
+}
 EMU_HD double rsqrt_n(double x) {
 #ifdef __CUDA_ARCH__
   if (mid_range(x)) {
@@ -71,6 +80,13 @@ EMU_HD double sqrt_n(double x) {
   }
 #endif
   return sqrt(x);
+}
+
+// Tangent of the Jacobi rotation that zeroes the entry apq of a symmetric
+// matrix with the diagonal entries app and aqq.
+EMU_HD double jacobi_tan(double app, double aqq, double apq) {
+  const double theta = div_n(aqq - app, 2.0 * apq);
+  return copysign(inv_n(fabs(theta) + sqrt_n(theta * theta + 1.0)), theta);
 }
 
 // ---------------------------------------------------------------- 3x3 ------
