@@ -390,8 +390,10 @@ size_t pcg64_smem(int rows, bool coarse) {
 
 template <int MAXT, bool C>
 cudaError_t launch64(const PcgArgsT<double>& args, int rows, int grid, int threads, cudaStream_t st) {
-  const size_t smem = pcg64_smem(rows, C);
-  if (smem > 40 * 1024) {  // with the static arrays above the default 48 KB: opt in once per device
+  // Every shape of an instantiation within one limit, raised once per device.
+  // (Static and dynamic bytes together decide: 13 to 14 KB of static arrays
+  // pass the default 48 KB with 192 rows without a coarse space already.)
+  {
     static bool set[64] = {false};
     static std::mutex mu;
     std::lock_guard<std::mutex> lock(mu);
@@ -406,6 +408,7 @@ cudaError_t launch64(const PcgArgsT<double>& args, int rows, int grid, int threa
       set[dev] = true;
     }
   }
+  const size_t smem = pcg64_smem(rows, C);
   PcgArgsT<double> a = args;
   int r = rows;
   void* params[] = {(void*)&a, (void*)&r};
