@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "emu.h"
+#include "emu_corners.h"
 #include "emu_internal.h"
 #include "emu_pcg.h"
 
@@ -113,13 +114,7 @@ extern "C" int emu_fiber_field(int64_t n_verts, const double* rest_pos, int64_t 
   // The Laplacian row by row: a vertex's tets in order, each neighbour's place
   // in the row remembered by vertex (a sort of all 16 m entries by key took
   // most of the call before).
-  std::vector<int32_t> sptr(n + 1, 0), slot(4 * m);
-  for (int64_t k = 0; k < 4 * m; ++k) ++sptr[tets[k] + 1];
-  for (int64_t v = 0; v < n; ++v) sptr[v + 1] += sptr[v];
-  {
-    std::vector<int32_t> at(sptr.begin(), sptr.end() - 1);
-    for (int64_t k = 0; k < 4 * m; ++k) slot[at[tets[k]]++] = (int32_t)k;
-  }
+  const VertexCorners vc = vertex_corners(n, m, tets);
   std::vector<double> rhs(3 * n, 0.0), dinv(n, 1.0), val;
   std::vector<int32_t> rowptr(n + 1, 0), col, place(n, -1);
   col.reserve(16 * n);
@@ -131,9 +126,9 @@ extern "C" int emu_fiber_field(int64_t n_verts, const double* rest_pos, int64_t 
       rowbuf.push_back({(int32_t)v, 1.0});
       rhs[3 * v] = (double)dir[v];
     } else {
-      for (int32_t k = sptr[v]; k < sptr[v + 1]; ++k) {
-        const int64_t i = slot[k] / 4;
-        const int a = slot[k] % 4;
+      for (CornerIndex k = vc.ptr[v]; k < vc.ptr[v + 1]; ++k) {
+        const int64_t i = vc.slot[k] / 4;
+        const int a = (int)(vc.slot[k] % 4);
         double gN[4][3];
         for (int r = 0; r < 3; ++r)
           for (int c = 0; c < 3; ++c) gN[r][c] = Dinv[(3 * r + c) * m + i];
