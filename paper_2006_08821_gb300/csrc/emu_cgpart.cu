@@ -121,6 +121,7 @@ bool build_cg_partition(int64_t n, const double* Q, const std::vector<int32_t>& 
       }
       std::sort(row.begin(), row.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
       P.rowptr[r + 1] = P.rowptr[r] + (int32_t)row.size();
+      P.row_max = std::max(P.row_max, (int)row.size());
       for (size_t k = 0; k < row.size(); ++k) {
         P.col.push_back(row[k].first);
         P.val.push_back((float)row[k].second);

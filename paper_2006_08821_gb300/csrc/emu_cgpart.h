@@ -21,6 +21,7 @@ constexpr int kChebMax = 8;  // largest polynomial degree of the local part
 struct CgPartHost {
   int G = 0, rpt = 0, nt = 0;
   int lw = 0;                      // local off-diagonal entries per row slot
+  int row_max = 0;                 // entries of the longest row of the permuted Laplacian
   int degree = 1;                  // polynomial degree (1: Jacobi only)
   std::vector<int32_t> perm;       // partition row -> vertex
   std::vector<int32_t> off;        // G + 1 row offsets of the parts
@@ -34,6 +35,17 @@ struct CgPartHost {
   float c0 = 1.f;                  // 1 / theta
   float c1[kChebMax] = {0}, c2[kChebMax] = {0};  // step i: d = c1 d + c2 res
 };
+
+// Whether the FP32 CG kernels gather a row's first 16 entries at once instead of
+// 8, from the matrix and from the local table (``lw`` entries per row): the rows
+// of a regular grid hold at most 7, those of an irregular mesh about 14, whose
+// entries beyond the eighth would run one dependent load at a time (59,840 tets,
+// degree 4: 4,000 -> 2,900 cycles for the SpMV of a CG iteration; the local
+// products, 9,300 cycles, are bound by shared-memory bank conflicts of the
+// 16-byte gathers either way). Without a local table (degree 1) the longest
+// row of the matrix decides.
+constexpr int kWideRows = 16, kNarrowRows = 8;
+inline bool cg_wide_rows(int lw, int row_max) { return (lw > 0 ? lw : row_max) > kNarrowRows; }
 
 // Largest number of local entries per row slot the pipelined kernel holds in
 // shared memory for ``rpt`` rows per thread.

@@ -103,6 +103,7 @@ struct emu_handle {
   float *cg_val = nullptr, *cg_dinv = nullptr, *cg_phi = nullptr, *cg_aphi = nullptr;
   uint32_t* cg_loc = nullptr;
   int cg_lw = 0, cg_degree = 1;
+  int row_max = 0, cg_row_max = 0;  // entries of the longest row: of the Laplacian, of the permuted one
   float cg_c0 = 1.f, cg_c1[kChebMax] = {0}, cg_c2[kChebMax] = {0};
   double cg_lmax = 0.0;            // Gershgorin bound of the local blocks (the polynomial's interval)
   int cg64_rows = 128;             // rows per block of the FP64 CG's generic kernel (grid_pcg3 = ceil(n / cg64_rows), capped)

@@ -189,6 +189,7 @@ cudaError_t run_pcg32(emu_handle* h, const float* rhs, float* x, double tol) {
     w.ug = h->ug32;
     w.part = h->part32;
     w.sync = h->sync32;
+    w.row_max = h->cg_part ? h->cg_row_max : h->row_max;
     if (h->cg_part) {
       // the partitioned system with the block-local preconditioner (b and x
       // stay in vertex order)
@@ -1109,6 +1110,7 @@ int emu_create(const emu_mesh_desc* desc, const emu_params* params, const emu_al
   h->device = dev;
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t nnz = (int64_t)colv.size();
+  for (int64_t v = 0; v < n; ++v) h->row_max = std::max(h->row_max, rowptr[v + 1] - rowptr[v]);
   // row partition and local preconditioner of the pipelined FP32 CG
   CgPartHost cgp;
   if (h->mixed) {
@@ -1117,6 +1119,7 @@ int emu_create(const emu_mesh_desc* desc, const emu_params* params, const emu_al
       h->cg_part = build_cg_partition(n, Q, rowptr, colv, valv, g32, r32, kPcg32Threads, prm.cg_local_degree, &cgp);
     if (h->cg_part) {
       h->cg_lw = cgp.lw;
+      h->cg_row_max = cgp.row_max;
       h->cg_degree = cgp.degree;
       h->cg_lmax = cgp.lmax;
       h->cg_c0 = cgp.c0;

@@ -90,6 +90,7 @@ struct Pcg32Work {
   const int32_t* off = nullptr;   // grid + 1 row offsets of the blocks' parts
   const uint32_t* loc = nullptr;  // local table: (grid x rpt x lw x 256) words
   int lw = 0;                     // local entries per row slot
+  int row_max = 0;                // entries of the longest row of args' matrix
   int cluster = 0;                // set by the launch: the grid is one cluster
   int degree = 1;                 // degree of the local polynomial (1: Jacobi)
   float c0 = 1.f;                 // Chebyshev coefficients (emu_cgpart.h)

@@ -34,13 +34,6 @@ namespace {
 constexpr int NT = kPcg32Threads;  // threads per block
 constexpr int NR = 3;    // right-hand sides (x, y, z)
 constexpr int kGather = 16;  // entries of a matrix row gathered at once
-// Entries gathered at once, from the pruned system and from the local table:
-// 8 where the local rows hold at most 8 (a regular grid's pruned rows hold 7),
-// 16 for the rows of an irregular mesh (about 14), whose entries beyond the
-// eighth used to run one dependent load at a time (59,840 tets: 4,000 -> 2,900
-// cycles for the SpMV of a CG iteration; the local products, 9,300 cycles, are
-// bound by shared-memory bank conflicts of the 16-byte gathers either way).
-constexpr int kWideRows = 16, kNarrowRows = 8;
 constexpr int kMaxGridStrides = 8;  // grid_sum_f handles up to 256 blocks
 // words of Pcg32Work::sync, one 128-byte line apart
 constexpr int kSyncCount = 0, kSyncDone = 32, kSyncErr = 64;
@@ -1147,7 +1140,7 @@ cudaError_t launch32w(const PcgArgsT<float>& args, const Pcg32Work& work, int gr
 template <int RPT, bool C>
 cudaError_t launch32(const PcgArgsT<float>& args, const Pcg32Work& work, int grid, cudaStream_t st) {
   if constexpr (RPT <= 4)
-    if (work.off && work.lw > kNarrowRows) return launch32w<RPT, C, true>(args, work, grid, st);
+    if (cg_wide_rows(work.off && work.degree > 1 ? work.lw : 0, work.row_max)) return launch32w<RPT, C, true>(args, work, grid, st);
   return launch32w<RPT, C, false>(args, work, grid, st);
 }
 }  // namespace
@@ -1198,7 +1191,7 @@ cudaError_t launch32p(const PcgArgsT<float>& args, const Pcg32Work& work, int gr
   Pcg32Work w = work;
   const int lw = w.degree > 1 ? w.lw : 0;
   if (lw > cg_local_width_max(RPT) || (w.degree > 1 && !w.loc)) return cudaErrorInvalidValue;
-  const void* f = w.lw > kNarrowRows ? (const void*)pcg32p_kernel<RPT, true> : (const void*)pcg32p_kernel<RPT, false>;
+  const void* f = cg_wide_rows(lw, w.row_max) ? (const void*)pcg32p_kernel<RPT, true> : (const void*)pcg32p_kernel<RPT, false>;
   return launch_blocks(f, grid, a, w, pipe_smem<RPT>(lw), st);
 }
 }  // namespace
