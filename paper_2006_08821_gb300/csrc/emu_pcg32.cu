@@ -1108,9 +1108,10 @@ constexpr size_t plain_smem(bool parted, int lw) {
 
 template <int RPT, bool C, bool W>
 cudaError_t prepare32() {
-  // above the default 48 KB the kernel needs the opt-in, a per-device attribute
+  // the largest shape's dynamic shared memory, a per-device attribute (with the
+  // static arrays even one row per thread passes the default 48 KB from 21
+  // local entries per row)
   const size_t smem = plain_smem<RPT, C>(RPT <= 4, RPT <= 4 ? cg_local_width_max(RPT) : 0);
-  if (smem <= 48 * 1024) return cudaSuccess;
   static bool set[64] = {false};
   static std::mutex mu;  // handles may be built from several threads
   std::lock_guard<std::mutex> lock(mu);
@@ -1174,7 +1175,6 @@ cudaError_t prepare32p() {
   static std::mutex mu;  // handles may be built from several threads
   std::lock_guard<std::mutex> lock(mu);
   const size_t smem = pipe_smem<RPT>(cg_local_width_max(RPT));
-  if (smem <= 48 * 1024) return cudaSuccess;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
