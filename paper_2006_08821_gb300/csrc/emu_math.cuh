@@ -21,11 +21,18 @@ namespace emu {
 
 template <typename T> EMU_HD T rsqrt2() { return T(0.70710678118654752440); }
 
-// 1 / x, 1 / sqrt(x), sqrt(x) in FP64. On the device Newton's iteration from the hardware's estimates (good to about
-// 2^-20; one cubic step leaves an ulp or so): a warp instruction of FP64 costs
-// its warp 64 cycles on GB300, and a division or square root is some twenty of
-// them where these take three to eight. Arguments near the ends of the range
-// (tested on the exponent bits) take the plain expressions.
+// 1 / x, 1 / sqrt(x), sqrt(x) in FP64. On the device one step of third order
+// from the hardware's estimate r of 1 / x or 1 / sqrt(x) (the approximate PTX
+// instructions, whose results carry 20 mantissa bits: relative error below
+// 2^-19). With e = 1 - x r, 1 / x = r (1 - e)^-1, and with e = 1 - x r^2,
+// 1 / sqrt(x) = r (1 - e)^-1/2: the binomial series of both to e^2 (the
+// hyperpower iteration; Householder's method of second order). The root is
+// Heron's step from x r, its residual x - s^2 formed by one fma. Errors, in
+// ulps, derived and measured over the whole range: 0.57 and 0.504, 1.16 and
+// 0.97, 0.51 and 0.5. Arguments outside 2^-500 .. 2^500 (tested on the exponent
+// bits), zeros, infinities and NaN take the plain expressions. A warp
+// instruction of FP64 costs its warp 64 cycles on GB300, and a division or a
+// root is some twenty of them where these take three to eight.
 EMU_HD bool positive_n(float x) { return x > 0.f; }
 EMU_HD bool positive_n(double x) {  // x > 0 (false for NaN), on the bits on the device
 #ifdef __CUDA_ARCH__
