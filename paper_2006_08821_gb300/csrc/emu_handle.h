@@ -401,35 +401,4 @@ template <> inline TetArgs<double> emu_handle::args<double>() {
   a.nu = has_force ? nu64 : nullptr;
   return a;
 }
-template <> inline TetArgs<float> emu_handle::args<float>() {
-  TetArgs<float> a;
-  a.m = m;
-  a.n = n;
-  a.tet = tet;
-  a.Dinv = Dinv;
-  a.V = V;
-  a.c = c;
-  a.w = w;
-  a.mu = mu;
-  a.lam = lam;
-  a.u = u;
-  a.ka = ka;
-  a.gam = gam32;
-  a.R = R;
-  a.s = s;
-  a.q = q;
-  a.dq = dq;
-  a.g = g;
-  a.y = y32;
-  a.d = d32;
-  a.Uw = Uw32;
-  a.contrib = contrib;
-  a.z = z;
-  a.sc = sc;
-  a.partials = part_grad;
-  a.tkind = tkind;
-  a.bone_st = bst;
-  a.nu = has_force ? nu64 : nullptr;
-  return a;
-}
 

@@ -1295,11 +1295,11 @@ int emu_set_external_forces(emu_handle* h, const double* f, int64_t n_verts) {
     EMU_CK(cudaMemcpyAsync(rhs, fb.data(), 24 * n, cudaMemcpyHostToDevice, h->st));
     EMU_CK(cudaMemsetAsync(x, 0, 24 * n, h->st));
     PcgArgsT<double> pa = h->pcg64(rhs, x, 1e-13);
-    // Mixed path: the generic kernel (it is the one without phit). A last-bit
+    // Mixed path: the generic kernel. A last-bit
     // change of nu moves its FP32 copy here and there, and a cantilever's
     // converged positions by up to 1e-5 of the mesh at 1e-6 (soft bending
     // modes), so a one-off solve is no place to change the rounding.
-    if (h->mixed) pa.phit = nullptr;
+    pa.generic = h->mixed;
     EMU_CK(launch_pcg<double>(3, pa, h->grid_pcg3, h->st));
     launch_nu(m, h->tet, h->Dinv, h->w, x, h->nu64, h->mixed ? h->nu32 : nullptr, h->st);
     EMU_CK(cudaGetLastError());

@@ -927,15 +927,10 @@ void launch_compose_F(int64_t m, const double* R, const double* s, double* F, cu
 
 // explicit instantiations
 template void launch_grad<double>(const TetArgs<double>&, int, int, cudaStream_t);
-template void launch_grad<float>(const TetArgs<float>&, int, int, cudaStream_t);
 template void launch_syrk<double>(const TetArgs<double>&, int, double*, cudaStream_t);
-template void launch_syrk<float>(const TetArgs<float>&, int, double*, cudaStream_t);
 template void launch_dir<double>(const TetArgs<double>&, int, int, cudaStream_t);
-template void launch_dir<float>(const TetArgs<float>&, int, int, cudaStream_t);
 template void launch_ls<double>(const TetArgs<double>&, int, int, const LsSelect&, cudaStream_t);
-template void launch_ls<float>(const TetArgs<float>&, int, int, const LsSelect&, cudaStream_t);
 template void launch_update_tets<double>(const TetArgs<double>&, int, int, double*, cudaStream_t);
-template void launch_update_tets<float>(const TetArgs<float>&, int, int, double*, cudaStream_t);
 template void launch_gamma<double>(int64_t, const int4*, const double*, const double*, double*, cudaStream_t);
 template void launch_gamma<float>(int64_t, const int4*, const double*, const double*, float*, cudaStream_t);
 

@@ -628,43 +628,9 @@ template <typename T> EMU_HD void apply_I_minus_N(const T* Uw, T* x) {
 // X <- (g X + X^-T / g) / 2 with determinant scaling g = |det X|^(-1/3)
 // (N. J. Higham, "Computing the polar decomposition, with applications",
 // SIAM J. Sci. Stat. Comput. 7, 1986). Returns the rotation in R and the
-// iteration count; ``tol`` bounds the Frobenius change of the last step.
-template <typename T> EMU_HD int polar_rotation(const T* X0, T* R, T tol, int max_iter) {
-  T X[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) X[i] = X0[i];
-  int it = 0;
-  for (; it < max_iter; ++it) {
-    T Xi[9];
-    T det = inv3(X, Xi);
-    T g = T(1);
-    if (it < 4) {
-      T ad = det > T(0) ? det : -det;
-      g = T(1) / cbrt(ad);
-    }
-    T ig = T(1) / g;
-    T diff = T(0);
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        T nx = T(0.5) * (g * X[3 * r + c] + ig * Xi[3 * c + r]);
-        T dd = nx - X[3 * r + c];
-        diff += dd * dd;
-        X[3 * r + c] = nx;
-      }
-    if (diff <= tol * tol && it >= 1) {
-      ++it;
-      break;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 9; ++i) R[i] = X[i];
-  return it;
-}
-
-// The same in FP64 without the scaling (a cube root and two divisions) near
-// det = 1, where the plain iteration converges in the same count.
+// iteration count; ``tol`` bounds the Frobenius change of the last step. The
+// scaling (a cube root and two divisions) is left out near det = 1, where the
+// plain iteration converges in the same count.
 EMU_HD int polar_rotation(const double* X0, double* R, double tol, int max_iter) {
   double X[9];
 #pragma unroll

@@ -56,7 +56,6 @@ struct MixArgs {
 
 void launch_grad_mixed(const MixArgs& a, int grid, cudaStream_t st);
 void launch_dir_mixed(const MixArgs& a, int grid, cudaStream_t st);
-// Line-search constants and the direction kernel's g.d partials, for the
 // Trial energies of one pass and, in its last block, the selected step
 // (ls_finish); the gradient kernel likewise leaves ||g||^2 in sc.
 void launch_ls_mixed(const MixArgs& a, int grid, const LsSelect& sel, cudaStream_t st);

@@ -507,7 +507,7 @@ int device_sms() {
 template <typename T> cudaError_t launch_pcg(int nrhs, const PcgArgsT<T>& args, int grid, cudaStream_t st) {
   if constexpr (std::is_same_v<T, double>) {
     int g64 = 0, rows = 0;
-    if (nrhs == 3 && (!args.phi || args.phit) && pcg64_shape(args.n, device_sms(), &g64, &rows))
+    if (nrhs == 3 && !args.generic && (!args.phi || args.phit) && pcg64_shape(args.n, device_sms(), &g64, &rows))
       return launch_pcg64(args, g64, rows, st);
     if (nrhs == 16) {
       const int columns = pcg16_columns(args.n, grid, device_sms());

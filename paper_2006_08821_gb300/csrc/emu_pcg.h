@@ -51,6 +51,7 @@ template <typename T> struct PcgArgsT {
   const T* phi;        // n x 16 coarse basis (null: Jacobi only; 3 columns only)
   const double* Einv;  // 16 x 16 (pseudo-)inverse of Phi^T L Phi
   const T* phit = nullptr;  // 16 x n: Phi T with T T^T = Einv, mode-major (FP64; null where phi is)
+  bool generic = false;     // three FP64 columns: the generic kernel whatever the size
   bool bar_clean = false;   // bar's v_ words are zero: no memset before a launch of pcg64_kernel
   unsigned long long wait_ns = kWaitLimitNs;  // limit of each grid-barrier wait
 };

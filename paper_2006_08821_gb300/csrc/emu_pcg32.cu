@@ -207,8 +207,9 @@ __device__ __forceinline__ void grid_sum_f(const float* __restrict__ part, int n
   __syncthreads();
 }
 
-// The rows vr[k] of a partitioned system (or of the whole one), and the same
-// product with their first GW entries gathered at once. With HOLD those
+// The matrix rows vr[k] of a partitioned system (or of the whole one) and their
+// product with a vector, the first GW entries of a row gathered at once and
+// the rest in a loop. With HOLD those
 // entries stay in registers for the whole launch: every grid barrier ends in
 // an acquire, which empties L1, so rereading them cost two L2 round trips
 // before the gather itself could start (2,000 of 14,500 cycles of a CG
