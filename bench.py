@@ -55,8 +55,11 @@ L2_BYTES = 129e6  # GB300 L2
 
 # DRAM bytes (read + write) per launch of a phase's kernel from one ncu
 # capture of the unchanged kernel (summaries under profiles/); left out once
-# the kernel has changed since (the CG, the gradient, the line search).
+# the kernel has changed since.
 NCU_TRAFFIC = {
+    "pcg": (18.21e6, "profiles/pcg32p_kernel_mtu401920.md"),
+    "grad": (124.27e6, "profiles/k_grad_m_mtu401920.md"),
+    "ls": (82.96e6, "profiles/k_ls_m_mtu401920.md"),
     "dir": (230.63e6, "profiles/k_dir_m_mtu401920.md"),
     "syrk": (183.30e6, "profiles/k_syrk05_mtu401920.md"),
 }

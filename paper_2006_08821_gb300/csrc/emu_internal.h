@@ -106,7 +106,7 @@ void set_last_error(const char* msg);
 // be placed and waits until its predecessor has completed and its writes are
 // visible (nothing without the attribute). Each block waits before it touches
 // memory, so the order of effects is that of plain launches. It hides launch
-// gaps where a kernel is a few blocks: 144 tets 101 -> 93 us per Newton
+// gaps where a kernel is a few blocks: 144 tets 101 -> 96 us per Newton
 // iteration. On larger meshes the waiting blocks take more than they give
 // (6,080 tets 124 -> 126 us, 401,920 tets 445 -> 472 us), so the launchers ask for
 // it up to kDepTets tets.

@@ -270,9 +270,9 @@ constexpr int kCapNB = 4;  // columns of a panel
 // entries are a prefix and whole warps drop out as it shrinks. In FP64 a warp
 // instruction holds an SM's FP64 pipe for 19 cycles: 1.1e4 cycles for the
 // updates, and the pivots' reciprocals are Newton steps in one warp.
-// Measured per Newton iteration with the reduction (phase times): FP32 27 us
-// as two launches with a barrier and a division per column, 19 us now; FP64 83
-// us, 33 us now.
+// Measured per Newton iteration with the reduction (event pairs around the
+// phase, which add about 4 us to a launch): FP32 27 us as two launches with a
+// barrier and a division per column, 20 to 22 us now; FP64 83 us, 34 us now.
 template <typename T>
 __global__ void __launch_bounds__(256) k_cap(const double* __restrict__ cpart, int nblk, double* __restrict__ cfull,
                                              const double* __restrict__ cadd, double* z, DevScalars* sc) {

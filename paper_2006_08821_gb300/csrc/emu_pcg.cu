@@ -13,7 +13,7 @@
 //
 // This is the generic kernel: any size, columns and precision. Three FP64
 // columns of up to 320 rows per SM and sixteen of up to 64 run the kernels of
-// emu_pcg64.cu (launch_pcg picks; 1.3 to 3 times faster there), the mixed path's
+// emu_pcg64.cu (launch_pcg picks; the times of both are there), the mixed path's
 // FP32 solves those of emu_pcg32.cu.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
